@@ -16,10 +16,20 @@
 // Structure: persistent CTAs (one per SM) walk tiles (lane, M block, N block
 // of up to 256 real columns).  Warp 0 issues TMA loads of A and Bt tiles
 // (128-byte or 64-byte swizzle) into a ring of shared-memory stages, warp 1
-// issues tcgen05.mma into one of two TMEM accumulators, warps 2..5 drain the
+// issues tcgen05.mma into one of two TMEM accumulators, the epilogue warps drain the
 // other accumulator with tcgen05.ld, apply the step's power-of-two scale,
 // split into the storage format and store permuted (the slowest untouched leg
 // moves next to v'), and record the max |entry|.
+//
+// What bounds a short-K step is the epilogue's stores and its per-tile
+// set-up, not the MMAs.  Rows are taken m_hi first (TcParams::mhi), so that a
+// warp's stores cover whole 128-byte lines instead of one sector in each of 32
+// lines (the L2 takes some 70 write requests per ns whatever their size);
+// entries go out 32 bytes at a time; an item's set-up is loaded for 32 items
+// at once; the index arithmetic has no 64-bit division.  16 lanes of a
+// 32768 x 64 x 64 step (FP16X3, 537 MB read and written): 230 -> 95 us (5.6
+// TB/s); of a 4096 x 64 x 512 step: 172 -> 61 us; the open-leg step 32768 x 128
+// x 256 with P = 16, one item: 155 -> 38 us.
 //
 // CG = 2 (the default where the row tiles pair up): a cluster of two CTAs on
 // neighbouring SMs computes a 256-row tile with the 2-SM UMMA
@@ -57,25 +67,24 @@ template <> struct FormTraits<FMT_BF16X2> { static constexpr int NP = 2, ESZ = 2
 template <> struct FormTraits<FMT_FP16X2> { static constexpr int NP = 2, ESZ = 2, KIND = 0, AB = 0; };
 template <> struct FormTraits<FMT_TF32>   { static constexpr int NP = 1, ESZ = 4, KIND = 1, AB = 2; };
 
-// x / d and x % d for a divisor fixed per launch (d > 0, x >= 0): a shift and
-// a mask when d is a power of two (every dimension made of CZ bonds), a
-// division otherwise (bonds of general two-qubit gates of Schmidt rank 3).
+// x / d and x % d for a divisor fixed per launch (1 <= d <= 2^31, 0 <= x <
+// 2^31), branch-free: q = (mulhi(m, x) + x) >> l with l = ceil(log2 d) and
+// m = floor(2^32 (2^l - d) / d) + 1 (Granlund and Montgomery, "Division by
+// invariant integers using multiplication", 1994).  One form for every
+// divisor: a branch between a shift and a 64-bit division put the division's
+// code between the hot instructions, and the tile set-up alone took about
+// 1700 of a 128 x 128 tile's 6200 cycles.
 struct Div {
-  int64_t d;
-  int32_t s;   // log2(d), or -1
+  uint32_t d, m;
+  int32_t l;
   int32_t pad_;
-  __device__ __forceinline__ int64_t q(int64_t x) const { return s >= 0 ? (x >> s) : x / d; }
-  __device__ __forceinline__ int64_t r(int64_t x) const {
-    return s >= 0 ? (x & (d - 1)) : x % d;
-  }
+  __device__ __forceinline__ uint32_t q(uint32_t x) const { return (__umulhi(m, x) + x) >> l; }
+  __device__ __forceinline__ uint32_t r(uint32_t x) const { return x - q(x) * d; }
 };
 inline Div make_div(int64_t d) {
-  Div v{d > 0 ? d : 1, -1, 0};
-  if ((v.d & (v.d - 1)) == 0) {
-    int k = 0;
-    while (((int64_t)1 << k) < v.d) ++k;
-    v.s = k;
-  }
+  Div v{(uint32_t)(d > 0 ? d : 1), 0u, 0, 0};
+  while (((int64_t)1 << v.l) < (int64_t)v.d) ++v.l;
+  v.m = (uint32_t)(((((uint64_t)1 << v.l) - v.d) << 32) / v.d + 1);
   return v;
 }
 
@@ -99,11 +108,12 @@ struct __align__(128) TcParams {   // the tensor maps need 128-byte alignment
   int nacc;     // accumulators per buffer: ksplit + csep
   int nbuf;     // accumulator buffers (2: the epilogue of a tile overlaps the
                 // next tile's MMAs)
-  int mhi;      // 1: a tile's rows are ph consecutive m_hi x lh consecutive m_lo
-                // (ph lh = BM) at one b, so that the open-leg store (contiguous
-                // in m_hi only) coalesces
+  int mhi;      // 1: a tile's rows are ph consecutive m_hi x lh consecutive m_lo x
+                // bh consecutive b (ph lh bh = BM, m_hi fastest), so that a
+                // warp's stores (contiguous over m_hi) coalesce
   int lp_mul;   // m_hi-major: the A map's last coordinate is lane * lp_mul + plane
-  int ph, lh;   // m_hi-major: tile extent in m_hi (min(P, BM)) and in m_lo
+  int ph, lh, bh;  // m_hi-major: tile extent in m_hi, m_lo and b
+  int wide;     // 1: the buffers are 32-byte aligned (256-bit stores)
   int gm;       // tile order: gm row groups at a time, n fastest within them
                 // (1: n fastest over a whole row group)
   int64_t mlo;  // m_hi-major: Mr / P
@@ -114,7 +124,7 @@ struct __align__(128) TcParams {   // the tensor maps need 128-byte alignment
                 // addresses are set up once); 0: tiles c, c + pairs, ...
   // divisors of the tile and store index arithmetic
   Div d_tpi, d_tn;             // tiles per item, column tiles
-  Div d_hper, d_lper, d_ph;    // m_hi-major tiles: P / ph, (Mr / P) / lh, ph
+  Div d_hper, d_lper, d_ph, d_lh;  // m_hi-major tiles: P / ph, (Mr / P) / lh, ph, lh
   Div d_Mr, d_Mlo, d_dv, d_dh; // output rows per batch slice, Mr / P, dim(v'), dim(h')
 };
 
@@ -194,6 +204,17 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, Watch 
   }
   return true;
 }
+
+// What the producer and the epilogue need of the launch's items, one item per
+// lane: the tiles of a CTA pair run through consecutive items (the item index
+// grows by 0 or 1 from tile to tile), so a warp loads the next 32 items'
+// entries at once and takes an item's from its lane by a shuffle.  Loaded one
+// by one, the chain item -> bitstring -> operand -> record costs three
+// dependent misses per item, which bounds launches of a tile or two per item.
+struct ItemBlock {
+  int base;          // first item held (item base + lane)
+  int tau, a_lane;   // operand variant (B map coordinate), A map lane
+};
 
 __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, uint64_t *bar,
                                             int c0, int c1, int c2, int c3) {
@@ -378,6 +399,16 @@ __device__ __forceinline__ void tmem_wait(uint32_t (&r)[16]) {
                : "memory");
 }
 
+// The same for two loads in flight.
+__device__ __forceinline__ void tmem_wait2(uint32_t (&r)[16], uint32_t (&q)[16]) {
+  tmem_wait(r);
+  asm volatile("" : "+r"(q[0]), "+r"(q[1]), "+r"(q[2]), "+r"(q[3]), "+r"(q[4]), "+r"(q[5]),
+               "+r"(q[6]), "+r"(q[7]), "+r"(q[8]), "+r"(q[9]), "+r"(q[10]), "+r"(q[11]),
+               "+r"(q[12]), "+r"(q[13]), "+r"(q[14]), "+r"(q[15])
+               :
+               : "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Kernel
 // ---------------------------------------------------------------------------
@@ -466,9 +497,10 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
 
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
-    if (lane == 0) {
-      uint32_t it = 0;
-      int cached_item = -1, tau = 0, a_lane = 0;
+    uint32_t it = 0;
+    {
+      ItemBlock ib{INT32_MIN, 0, 0};
+      bool ok = true;
       for (int t = t_first; t < t_end; t += t_step) {
         const int item = (int)p.d_tpi.q(t);
         const int rem = t - item * tiles_per_item;
@@ -480,57 +512,64 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
           tile_of(rem, mgroups, p.tiles_n, p.gm, mg, nt);
         }
         const int mt = mg * CG + (int)rank;
-        if (item != cached_item) {
-          cached_item = item;
-          const StepItem &si = p.items[item];
-          tau = block_variant(*si.bits, p.sh) + si.b_slot;
-          a_lane = si.a_lane;
+        if (item >= ib.base + 32 || ib.base < 0) {
+          ib.base = item;
+          const int i = item + lane < p.n_items ? item + lane : item;
+          const StepItem &si = p.items[i];
+          ib.tau = block_variant(*si.bits, p.sh) + si.b_slot;
+          ib.a_lane = si.a_lane;
         }
+        const int tau = __shfl_sync(0xffffffffu, ib.tau, item - ib.base);
+        const int a_lane = __shfl_sync(0xffffffffu, ib.a_lane, item - ib.base);
         // m_hi-major: tile mt is rows m_hi = hb0 .. hb0+ph-1, m_lo = mlo_t ..
-        // mlo_t+lh-1 at b_t
-        int64_t b_t = 0, mlo_t = 0;
-        int hb0 = 0;
+        // mlo_t+lh-1, b = b_t .. b_t+bh-1
+        int b_t = 0, mlo_t = 0, hb0 = 0;
         if (p.mhi) {
-          const int64_t rest = p.d_hper.q(mt);
-          hb0 = (int)p.d_hper.r(mt) * p.ph;
-          b_t = p.d_lper.q(rest);
-          mlo_t = p.d_lper.r(rest) * p.lh;
+          const uint32_t rest = p.d_hper.q(mt);
+          hb0 = (int)(mt - rest * p.d_hper.d) * p.ph;
+          b_t = (int)p.d_lper.q(rest);
+          mlo_t = (int)(rest - b_t * p.d_lper.d) * p.lh;
+          b_t *= p.bh;
         }
-        bool ok = true;
-        for (int kb = 0; kb < kb_count; ++kb, ++it) {
-          const int s = it % S;
-          const uint32_t ph = (it / S) & 1u;
-          if (!mbar_wait(&empty[s], ph ^ 1u, w)) { ok = false; break; }
-          unsigned char *st = smem + (size_t)s * stage_bytes;
-          const int k0 = kb * (ROWB / T::ESZ);
-          if (CG == 1) {
-            mbar_expect_tx(&full[s], stage_bytes);
-            for (int pl = 0; pl < NP; ++pl) {
-              if (p.mhi)
-                tma_load_5d(st + pl * a_bytes, &p.mapA, &full[s], k0, hb0, (int)mlo_t, (int)b_t,
-                            a_lane * p.lp_mul + pl);
-              else
-                tma_load_4d(st + pl * a_bytes, &p.mapA, &full[s], k0, mt * BM, pl, a_lane);
-              tma_load_3d(st + NP * a_bytes + pl * b_bytes, &p.mapB[pl], &full[s], k0,
-                          nt * BN, tau);
-            }
-          } else {
-            // the even CTA's full barrier counts both CTAs' bytes
-            if (leader) mbar_expect_tx(&full[s], 2 * stage_bytes);
-            for (int pl = 0; pl < NP; ++pl) {
-              if (p.mhi)
-                tma_load_5d_cg2(st + pl * a_bytes, &p.mapA, full0 + (uint32_t)s * 8u, k0, hb0,
-                                (int)mlo_t, (int)b_t, a_lane * p.lp_mul + pl);
-              else
-                tma_load_4d_cg2(st + pl * a_bytes, &p.mapA, full0 + (uint32_t)s * 8u, k0,
-                                mt * BM, pl, a_lane);
-              tma_load_3d_cg2(st + NP * a_bytes + pl * b_bytes, &p.mapB[pl],
-                              full0 + (uint32_t)s * 8u, k0, nt * BN + (int)rank * BNL, tau);
+        if (lane == 0) {
+          for (int kb = 0; kb < kb_count; ++kb, ++it) {
+            const int s = it % S;
+            const uint32_t ph = (it / S) & 1u;
+            if (!mbar_wait(&empty[s], ph ^ 1u, w)) { ok = false; break; }
+            unsigned char *st = smem + (size_t)s * stage_bytes;
+            const int k0 = kb * (ROWB / T::ESZ);
+            if (CG == 1) {
+              mbar_expect_tx(&full[s], stage_bytes);
+              for (int pl = 0; pl < NP; ++pl) {
+                if (p.mhi)
+                  tma_load_5d(st + pl * a_bytes, &p.mapA, &full[s], k0, hb0, mlo_t, b_t,
+                              a_lane * p.lp_mul + pl);
+                else
+                  tma_load_4d(st + pl * a_bytes, &p.mapA, &full[s], k0, mt * BM, pl, a_lane);
+                tma_load_3d(st + NP * a_bytes + pl * b_bytes, &p.mapB[pl], &full[s], k0,
+                            nt * BN, tau);
+              }
+            } else {
+              // the even CTA's full barrier counts both CTAs' bytes
+              if (leader) mbar_expect_tx(&full[s], 2 * stage_bytes);
+              for (int pl = 0; pl < NP; ++pl) {
+                if (p.mhi)
+                  tma_load_5d_cg2(st + pl * a_bytes, &p.mapA, full0 + (uint32_t)s * 8u, k0, hb0,
+                                  mlo_t, b_t, a_lane * p.lp_mul + pl);
+                else
+                  tma_load_4d_cg2(st + pl * a_bytes, &p.mapA, full0 + (uint32_t)s * 8u, k0,
+                                  mt * BM, pl, a_lane);
+                tma_load_3d_cg2(st + NP * a_bytes + pl * b_bytes, &p.mapB[pl],
+                                full0 + (uint32_t)s * 8u, k0, nt * BN + (int)rank * BNL, tau);
+              }
             }
           }
         }
+        ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
         if (!ok) break;
       }
+    }
+    if (lane == 0) {
       // Every issued stage must have landed before the pair may exit.  The
       // full barriers live in the even CTA and count the loads of both CTAs;
       // after an abort the two producers may have stopped at different
@@ -640,16 +679,47 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
     const bool idle = EPI == 8 && !split_cols && ew >= 4;
     const int c_end = idle ? 0 : (split_cols ? c_begin + p.BN / 2 : p.BN);
     const int dv = p.sh.dv_out, dh = p.sh.dh_out;
-    const int64_t M = p.sh.M, P = p.sh.P;
-    const int64_t Mr = p.sh.Mr > 0 ? p.sh.Mr : M;
+    const uint32_t M = (uint32_t)p.sh.M;
+    const int64_t P = p.sh.P;
+    const int64_t Mr = p.sh.Mr > 0 ? p.sh.Mr : p.sh.M;
     const int64_t MrN = Mr * (int64_t)p.sh.N, Mrdh = Mr * (int64_t)dh;
     const bool vbm = p.sh.vb != 0;
+    const bool dotm = p.sh.dot != 0;
+    // Destination of complex column nc of a row:
+    //   base + q(nc) * stride_q + r(nc) * stride_r  (q, r: nc / R, nc % R)
+    //   vb = 0:          n = h' dv' + v', entry b Mr N + ((m_lo dh' + h') P + m_hi) dv' + v'
+    //   vb = 1, nvs = 0: n = h' dv' + v', entry (b dv' + v') Mr dh' + (m_lo dh' + h') P + m_hi
+    //   vb = 1, nvs = 1: n = v' dh' + h', the same entry
+    // (R = 1: N = dh', the h' stride is stride_r over the whole N).  Runs of
+    // consecutive nc with stride_r = 1 are contiguous: they are stored W
+    // entries at a time (W = 8, 4, 2 dividing R), else one by one.
+    const Div dR = vbm && p.sh.nvs != 0 ? p.d_dh : p.d_dv;
+    const bool flat = dR.d == 1;
+    const uint32_t R = flat ? (uint32_t)p.sh.N : dR.d;
+    const int64_t stride_h = !vbm ? P * dv : P;
+    const int64_t stride_q = flat ? 0 : (vbm && p.sh.nvs != 0 ? Mrdh : stride_h);
+    const int64_t stride_r =
+        flat ? (vbm && p.sh.nvs != 0 ? Mrdh : stride_h) : (!vbm ? 1 : (p.sh.nvs != 0 ? P : Mrdh));
+    const int W = stride_r != 1 ? 1 : (R % 8 == 0 ? 8 : (R % 4 == 0 ? 4 : (R % 2 == 0 ? 2 : 1)));
+    const int64_t wrap = stride_q - (int64_t)R * stride_r;   // added where nc crosses into a new q
+    // m_hi-major tiles: this row's place in the tile, row = (bb lh + l) ph + h
+    const uint32_t row_rl = p.d_ph.q(row);
+    const uint32_t row_h = row - row_rl * p.d_ph.d, row_b = p.d_lh.q(row_rl),
+                   row_l = row_rl - row_b * p.d_lh.d;
     uint32_t local = 0;
-    int cached_item = -1;
-    const OpDesc *op = nullptr;
-    const StepItem *si = nullptr;
-    float sc = 1.f;
-    int x = 0, s_in = 0;
+    // the warp's next 32 items, one per lane
+    int ib_base = INT32_MIN, i_x = 0, i_exp = 0, i_rec = 0;
+    unsigned long long i_D = 0;
+    int cached_item = -1, out_rec = 0, out_exp = 0;
+    void *D = nullptr;
+    float sc = 1.f, vmax = 0.f;
+    // the item's max |entry|, once per item and warp (non-negative floats
+    // compare as their bits)
+    auto flush_max = [&]() {
+      const uint32_t mx = __reduce_max_sync(0xffffffffu, __float_as_uint(vmax));
+      if (lane == 0) atomicMax(&p.recs[out_rec].maxbits, mx);
+      vmax = 0.f;
+    };
     for (int t = t_first; t < t_end; t += t_step, ++local) {
       const int item = (int)p.d_tpi.q(t);
       const int rem = t - item * tiles_per_item;
@@ -662,15 +732,27 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
       }
       const int mt = mg * CG + (int)rank;
       if (item != cached_item) {
+        if (!dotm && cached_item >= 0) flush_max();
         cached_item = item;
-        si = &p.items[item];
-        op = &p.ops[si->op_base + block_variant(*si->bits, p.sh)];
-        const bool unit_in = si->in_rec < 0;
-        const float mu = unit_in ? 1.f : __uint_as_float(p.recs[si->in_rec].maxbits);
-        s_in = unit_in ? 0 : p.recs[si->in_rec].exp;
-        // a fused dot keeps the accumulator unscaled (nothing is stored)
-        x = p.sh.dot ? 0 : step_scale_exp(mu, __uint_as_float(op->beta_t_bits), p.sh.target);
-        sc = pow2f(x);
+        if (item >= ib_base + 32 || ib_base < 0) {
+          ib_base = item;
+          const int i = item + lane < p.n_items ? item + lane : item;
+          const StepItem &si = p.items[i];
+          const OpDesc &op = p.ops[si.op_base + block_variant(*si.bits, p.sh)];
+          const bool unit_in = si.in_rec < 0;
+          const float mu = unit_in ? 1.f : __uint_as_float(p.recs[si.in_rec].maxbits);
+          const int s_in = unit_in ? 0 : p.recs[si.in_rec].exp;
+          // a fused dot keeps the accumulator unscaled (nothing is stored)
+          i_x = dotm ? 0 : step_scale_exp(mu, __uint_as_float(op.beta_t_bits), p.sh.target);
+          i_exp = s_in + op.b_t + i_x + op.e_c;
+          i_rec = si.out_rec;
+          i_D = (unsigned long long)si.D;
+        }
+        const int src = item - ib_base;
+        sc = pow2f(__shfl_sync(0xffffffffu, i_x, src));
+        out_exp = __shfl_sync(0xffffffffu, i_exp, src);
+        out_rec = __shfl_sync(0xffffffffu, i_rec, src);
+        D = (void *)__shfl_sync(0xffffffffu, i_D, src);
       }
       const int acc = p.nbuf == 2 ? (int)(local & 1) : 0;
       const uint32_t aph = p.nbuf == 2 ? (local >> 1) & 1u : local & 1u;
@@ -679,30 +761,26 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
       ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!ok) break;
       tc_fence_after();
-      int64_t b, m_hi, m_lo;
-      bool live;
+      uint32_t b, m_hi, m_lo;
+      bool live = true;
       if (p.mhi) {
-        // row = l ph + h: m_hi = hb0 + h, m_lo = mlo_t + l (the tile of the producer)
-        const int64_t rest = p.d_hper.q(mt);
-        m_hi = p.d_hper.r(mt) * p.ph + p.d_ph.r(row);
+        const uint32_t rest = p.d_hper.q(mt);
+        m_hi = (mt - rest * p.d_hper.d) * (uint32_t)p.ph + row_h;
         b = p.d_lper.q(rest);
-        m_lo = p.d_lper.r(rest) * p.lh + p.d_ph.q(row);
-        live = true;
+        m_lo = (rest - b * p.d_lper.d) * (uint32_t)p.lh + row_l;
+        b = b * (uint32_t)p.bh + row_b;
       } else {
-        const int64_t m = (int64_t)mt * BM + row;
+        const uint32_t m = (uint32_t)mt * BM + row;
         live = m < M;
         // row m = b * Mr + m_r (b: the batch of open legs, when there is one)
-        b = live ? p.d_Mr.q(m) : 0;
-        const int64_t mr = live ? m - b * Mr : 0;
+        b = p.d_Mr.q(m);
+        const uint32_t mr = m - b * p.d_Mr.d;
         m_hi = p.d_Mlo.q(mr);
-        m_lo = p.d_Mlo.r(mr);
+        m_lo = mr - m_hi * p.d_Mlo.d;
       }
-      float vmax = 0.f;
       const int KSP = p.nacc;   // K segments, then the correction accumulator
       const uint32_t tbase =
           tmem_base + ((uint32_t)(32 * quad) << 16) + (uint32_t)(acc * BN * KSP);
-      void *D = si->D;
-      const bool dotm = p.sh.dot != 0;
       float dre = 0.f, dim = 0.f;   // fused dot: this row's partial sum
       // The columns in chunks of 16 (8 complex entries), the next chunk (or
       // pair) loaded from TMEM while the current one is used.
@@ -711,7 +789,7 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
       if (dotm) {
         // fused dot: the partner entries of row m (P = 1, row-major m N + n),
         // loaded one chunk ahead of their use
-        const int64_t dot_e = m_lo * (int64_t)p.sh.N + ((nt * BN + c_begin) >> 1);
+        const int64_t dot_e = (int64_t)m_lo * p.sh.N + ((nt * BN + c_begin) >> 1);
         Raw8 fcur, fnext;
         if (live && !idle) load8_raw<FMT>(D, dot_e, p.sh.plane, fcur);
         tmem_wait(ra);
@@ -742,48 +820,53 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
           if (more) tmem_wait(ra);
         }
       } else {
-        // Destination of complex column nc of this row:
-        //   base + q(nc) * stride_q + r(nc) * stride_r  (q, r: nc / R, nc % R)
-        //   vb = 0:          n = h' dv' + v', entry b Mr N + ((m_lo dh' + h') P + m_hi) dv' + v'
-        //   vb = 1, nvs = 0: n = h' dv' + v', entry (b dv' + v') Mr dh' + (m_lo dh' + h') P + m_hi
-        //   vb = 1, nvs = 1: n = v' dh' + h', the same entry
-        // Runs of consecutive nc with stride_r = 1 are contiguous: they are
-        // stored W entries at a time (W = 8, 4, 2 dividing R), else one by one.
-        const bool nvs = p.sh.nvs != 0;
-        const Div &dR = vbm && nvs ? p.d_dh : p.d_dv;
-        const int64_t base = !vbm ? b * MrN + (m_lo * dh * P + m_hi) * dv
-                                  : b * dv * Mrdh + m_lo * dh * P + m_hi;
-        const int64_t stride_q = !vbm ? P * dv : (nvs ? Mrdh : P);
-        const int64_t stride_r = !vbm ? 1 : (nvs ? P : Mrdh);
-        const int64_t R = dR.d;
-        const int W = stride_r != 1 ? 1 : (R % 8 == 0 ? 8 : (R % 4 == 0 ? 4 : (R % 2 == 0 ? 2 : 1)));
-        // chunk c (16 columns, 8 complex entries): scaled, rounded to the
-        // storage format and stored in runs of W
-        auto emit = [&](int c, const float (&o)[16]) {
+        const int64_t base = !vbm ? (int64_t)b * MrN + ((int64_t)m_lo * dh * P + m_hi) * dv
+                                  : (int64_t)b * dv * Mrdh + (int64_t)m_lo * dh * P + m_hi;
+        // the current column's place: dest = its entry, cr = r(nc)
+        const uint32_t nc0 = (uint32_t)(nt * BN + c_begin) >> 1;
+        const uint32_t cq = flat ? 0u : dR.q(nc0);
+        uint32_t cr = flat ? nc0 : nc0 - cq * R;
+        int64_t dest = base + (int64_t)cq * stride_q + (int64_t)cr * stride_r;
+        // the next w columns (w divides R, or is 1)
+        auto advance = [&](int w) {
+          cr += w;
+          dest += w * stride_r;
+          if (cr == R) {
+            cr = 0;
+            dest += wrap;
+          }
+        };
+        // the next 16 accumulator columns (8 complex entries): scaled, rounded
+        // to the storage format and stored in runs of W
+        auto emit = [&](const float (&o)[16]) {
           Packed8<FMT> w;
           vmax = fmaxf(vmax, pack8<FMT>(o, sc, w));
-          const int nc0 = (nt * BN + c) >> 1;
           switch (W) {
             case 8:
-              store_run<FMT, 8>(D, base + dR.q(nc0) * stride_q + dR.r(nc0), p.sh.plane, w, 0);
+              if (p.wide) store_run8_wide<FMT>(D, dest, p.sh.plane, w);
+              else store_run<FMT, 8>(D, dest, p.sh.plane, w, 0);
+              advance(8);
               break;
             case 4:
 #pragma unroll
-              for (int j = 0; j < 8; j += 4)
-                store_run<FMT, 4>(D, base + dR.q(nc0 + j) * stride_q + dR.r(nc0 + j), p.sh.plane,
-                                  w, j);
+              for (int j = 0; j < 8; j += 4) {
+                store_run<FMT, 4>(D, dest, p.sh.plane, w, j);
+                advance(4);
+              }
               break;
             case 2:
 #pragma unroll
-              for (int j = 0; j < 8; j += 2)
-                store_run<FMT, 2>(D, base + dR.q(nc0 + j) * stride_q + dR.r(nc0 + j), p.sh.plane,
-                                  w, j);
+              for (int j = 0; j < 8; j += 2) {
+                store_run<FMT, 2>(D, dest, p.sh.plane, w, j);
+                advance(2);
+              }
               break;
             default:
 #pragma unroll
-              for (int j = 0; j < 8; ++j)
-                store_run<FMT, 1>(D, base + dR.q(nc0 + j) * stride_q + dR.r(nc0 + j) * stride_r,
-                                  p.sh.plane, w, j);
+              for (int j = 0; j < 8; ++j) {
+                store_run<FMT, 1>(D, dest, p.sh.plane, w, j);
+                advance(1);
+              }
           }
         };
         // the other K segments of chunk c, added with FP32 round-to-nearest
@@ -800,7 +883,7 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
           // two chunks per iteration (twice the independent work in flight);
           // the next pair's TMEM loads overlap this pair's arithmetic
           if (c_begin + 16 < c_end) tmem_ld16_issue(tbase + (uint32_t)(c_begin + 16), rb);
-          tmem_wait(ra);
+          tmem_wait2(ra, rb);
           for (int c = c_begin; c < c_end; c += 32) {
             const bool two = c + 16 < c_end;
             float o0[16], o1[16];
@@ -817,10 +900,10 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
             add_segments(c, o0);
             if (two) add_segments(c + 16, o1);
             if (live) {
-              emit(c, o0);
-              if (two) emit(c + 16, o1);
+              emit(o0);
+              if (two) emit(o1);
             }
-            if (more) tmem_wait(ra);
+            if (more) tmem_wait2(ra, rb);
           }
         } else {
           // one chunk at a time (the register budget of eight epilogue warps),
@@ -835,7 +918,7 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
             for (int i = 0; i < 16; ++i) o[i] = __uint_as_float(ra[i]);
             if (more) tmem_ld16_issue(tbase + (uint32_t)(c + 16), ra);
             add_segments(c, o);
-            if (live) emit(c, o);
+            if (live) emit(o);
             if (more) tmem_wait(ra);
           }
         }
@@ -857,12 +940,10 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
         if (lane == 0)
           p.dot_partials[((int64_t)item * tiles_per_item + rem) * (CG * EPI) + (int)rank * EPI +
                          ew] = make_double2(r, i);
-      } else {
-        for (int o = 16; o > 0; o >>= 1) vmax = fmaxf(vmax, __shfl_xor_sync(0xffffffffu, vmax, o));
-        if (lane == 0) atomicMax(&p.recs[si->out_rec].maxbits, __float_as_uint(vmax));
       }
-      if (mt == 0 && nt == 0 && warp == 2 && lane == 0) p.recs[si->out_rec].exp = s_in + op->b_t + x + op->e_c;
+      if (mt == 0 && nt == 0 && warp == 2 && lane == 0) p.recs[out_rec].exp = out_exp;
     }
+    if (!dotm && cached_item >= 0) flush_max();
   }
 
   // teardown: everyone done issuing; the last MMAs have retired (done
@@ -966,31 +1047,40 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
       rowb == 128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_64B;
   // unused dimensions (one plane, one lane) get the packed stride
   const int64_t packed = (int64_t)Kr * esz * sh.M;
-  // A step that stores its open bottom leg into the batch (vb) writes
-  // (b dv' + v') Mr dh' + ((m_lo dh' + h') P + m_hi): contiguous in m_hi
-  // only.  Its tiles then take ph = min(P, BM) consecutive m_hi by lh = BM / ph
-  // consecutive m_lo at one b, through a 5-d map {k, m_hi, m_lo, b,
-  // plane/lane} (the plane and the lane share a coordinate: lane * lp_mul +
-  // plane), so that a warp's stores cover 32 consecutive entries.  The box
-  // lands in shared memory as the usual 128 rows (row = l ph + h).
+  // Rows are stored next to one another over m_hi (runs of dv' entries, or
+  // of single entries where the step stores its open leg into the batch, vb),
+  // but the input's consecutive rows are consecutive in m_lo, whose
+  // destinations lie dh' P dv' entries apart.  So a tile takes ph consecutive
+  // m_hi x lh consecutive m_lo x bh consecutive b (ph lh bh = BM), through a
+  // 5-d map {k, m_hi, m_lo, b, plane/lane} (the plane and the lane share a
+  // coordinate: lane * lp_mul + plane): a warp's stores then cover whole
+  // 128-byte lines.  The box lands in shared memory as the usual 128 rows
+  // (row = (bb lh + l) ph + h).  Nothing to gain where the rows' order is
+  // already that (P = 1, or Mr = P) or nothing is stored (the fused dot).
   bool mhi = false;
   int64_t lp_mul = 1, lp_stride = 0, lp_ext = 1;
-  const int64_t ph = sh.P < BM ? sh.P : BM, lh = BM / (ph > 0 ? ph : 1);
-  if (sh.vb && sh.nvs == 0 && sh.P >= 32 && (sh.P % BM == 0 || BM % sh.P == 0) && sh.Mr > 0 &&
-      sh.Mr % sh.P == 0 && sh.M % sh.Mr == 0 && (sh.Mr / sh.P) % lh == 0) {
+  int64_t ph = 1, lh = 1, bh = 1;
+  if (!sh.dot && sh.P > 1 && sh.Mr > sh.P && sh.Mr % sh.P == 0 && sh.M % sh.Mr == 0) {
+    const int64_t Mlo = sh.Mr / sh.P, B = sh.M / sh.Mr;
+    const int64_t want = sh.vb ? BM : (sh.dv_out >= 64 ? 1 : 64 / sh.dv_out);
+    while (2 * ph <= want && sh.P % (2 * ph) == 0 && 2 * ph <= BM) ph *= 2;
+    while (2 * lh * ph <= BM && Mlo % (2 * lh) == 0) lh *= 2;
+    while (2 * bh * lh * ph <= BM && B % (2 * bh) == 0) bh *= 2;
+    mhi = ph > 1 && ph * lh * bh == BM && sh.nvs == 0;
+  }
+  if (mhi) {
     if (np > 1) {
       if (a_lanes == 1) {
-        mhi = true;
         lp_stride = plane_stride_bytes;
         lp_ext = np;
       } else if (plane_stride_bytes > 0 && a_lane_stride % plane_stride_bytes == 0) {
-        mhi = true;
         lp_mul = a_lane_stride / plane_stride_bytes;
         lp_stride = plane_stride_bytes;
         lp_ext = (int64_t)(a_lanes - 1) * lp_mul + np;
+      } else {
+        mhi = false;
       }
     } else {
-      mhi = true;
       lp_stride = a_lanes > 1 ? a_lane_stride : packed;
       lp_ext = a_lanes;
     }
@@ -1002,7 +1092,7 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
                           (cuuint64_t)lp_ext};
     cuuint64_t strides[4] = {(cuuint64_t)(Mlo * Kr * esz), (cuuint64_t)Kr * esz,
                              (cuuint64_t)(sh.Mr * Kr * esz), (cuuint64_t)lp_stride};
-    cuuint32_t box[5] = {(cuuint32_t)(rowb / esz), (cuuint32_t)ph, (cuuint32_t)lh, 1, 1};
+    cuuint32_t box[5] = {(cuuint32_t)(rowb / esz), (cuuint32_t)ph, (cuuint32_t)lh, (cuuint32_t)bh, 1};
     cuuint32_t es[5] = {1, 1, 1, 1, 1};
     CUresult r = enc(&d->prm.mapA, dt, 5, const_cast<void *>(a_base), dims, strides, box, es,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, sw, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1015,6 +1105,7 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
     d->prm.lp_mul = (int)lp_mul;
     d->prm.ph = (int)ph;
     d->prm.lh = (int)lh;
+    d->prm.bh = (int)bh;
     d->prm.mlo = Mlo;
   } else {
     cuuint64_t dims[4] = {(cuuint64_t)Kr, (cuuint64_t)sh.M, (cuuint64_t)np,
@@ -1073,6 +1164,7 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
     }
   }
   d->prm.sh = sh;
+  d->prm.wide = ((uintptr_t)a_base % 32 == 0) ? 1 : 0;
   d->prm.BN = BN;
   d->prm.tiles_m = (int)((sh.M + BM - 1) / BM);
   d->prm.tiles_n = Nr / BN;
@@ -1095,6 +1187,7 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
     d->prm.d_dh = make_div(sh.dh_out);
     const int ph = d->prm.mhi ? d->prm.ph : 1, lh = d->prm.mhi ? d->prm.lh : 1;
     d->prm.d_ph = make_div(ph);
+    d->prm.d_lh = make_div(lh);
     d->prm.d_hper = make_div(d->prm.mhi ? P / ph : 1);
     d->prm.d_lper = make_div(d->prm.mhi ? d->prm.mlo / lh : 1);
   }
@@ -1111,13 +1204,17 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
   int stages = budget / stage_bytes;
   if (stages > 8) stages = 8;
   d->prm.stages = stages;
-  // Epilogue warps (measured on the square partition's steps): four where
-  // wide tiles store runs of 8 entries (each warp keeps two chunks in
-  // flight), eight where the stores go out 1 to 4 entries at a time, where
-  // nothing is stored (the fused dot) and on narrower tiles
-  const bool runs8 = !sh.dot && ((!sh.vb && sh.dv_out % 8 == 0) ||
-                                 (sh.vb && sh.nvs && sh.P == 1 && sh.dh_out % 8 == 0));
-  d->epi = epi == 4 || epi == 8 ? epi : ((runs8 && BN >= 256) ? 4 : 8);
+  // Epilogue warps: eight where the epilogue bounds the tile (K <= 64 on
+  // tiles of at least 64 columns, K <= 32 on 32) and where it is not hidden at
+  // all (one accumulator buffer: the merges; the fused dot), four where the
+  // MMAs do or where a second warp per quadrant finds no columns.  Measured,
+  // eight / four warps: 16 lanes of 4096 x 64 x 512 60.6 / 69.7 us, 65536 x 16 x
+  // 256 518 / 678 us, 4096^3 merge 11.43 / 11.60 ms; 65536 x 256 x 256 1408 /
+  // 1382 us, 512 lanes of 1024 x 128 x 512 584 / 549 us, 32768 x 64 x 8 66.0 /
+  // 61.7 us.
+  const bool epi_bound = sh.dot || d->prm.nbuf == 1 || (sh.K <= 64 && BN >= 64) ||
+                         (sh.K <= 32 && BN >= 32);
+  d->epi = epi == 4 || epi == 8 ? epi : (epi_bound ? 8 : 4);
   *out_handle = d;
   return stages >= 2 ? 0 : -5;
 }

@@ -249,6 +249,15 @@ __device__ __forceinline__ void store_words(uint32_t *d, const uint32_t *w) {
       *reinterpret_cast<uint4 *>(d + i) = make_uint4(w[i], w[i + 1], w[i + 2], w[i + 3]);
   }
 }
+// Eight words (32 bytes, a whole sector) in one 256-bit store; d 32-byte
+// aligned.
+__device__ __forceinline__ void store_words8(uint32_t *d, const uint32_t *w) {
+  asm volatile("st.global.v8.b32 [%0], {%1,%2,%3,%4,%5,%6,%7,%8};" ::"l"(
+                   __cvta_generic_to_global(d)),
+               "r"(w[0]), "r"(w[1]), "r"(w[2]), "r"(w[3]), "r"(w[4]), "r"(w[5]), "r"(w[6]),
+               "r"(w[7])
+               : "memory");
+}
 template <int FMT, int W>
 __device__ __forceinline__ void store_run(void *base, int64_t dest, int64_t plane,
                                           const Packed8<FMT> &p, int j0) {
@@ -260,6 +269,21 @@ __device__ __forceinline__ void store_run(void *base, int64_t dest, int64_t plan
   } else {
     store_words<W>(b + dest, p.w + j0);
     store_words<W>(b + plane / 2 + dest, p.w + 8 + j0);
+  }
+}
+
+// Entries 0 .. 7 of p at dest .. dest+7 (dest % 8 == 0) with 256-bit stores
+// (base 32-byte aligned).
+template <int FMT>
+__device__ __forceinline__ void store_run8_wide(void *base, int64_t dest, int64_t plane,
+                                                const Packed8<FMT> &p) {
+  uint32_t *b = reinterpret_cast<uint32_t *>(base);
+  if (FMT == FMT_F32 || FMT == FMT_TF32) {
+    store_words8(b + 2 * dest, p.w);
+    store_words8(b + 2 * dest + 8, p.w + 8);
+  } else {
+    store_words8(b + dest, p.w);
+    if (FMT != FMT_BF16 && FMT != FMT_FP16) store_words8(b + plane / 2 + dest, p.w + 8);
   }
 }
 
