@@ -671,13 +671,13 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
     // while chunk c is scaled, split and stored.
     const int quad = warp & 3;
     const int row = 32 * quad + lane;
-    // EPI = 8: warps ew and ew + 4 share a quadrant and split its columns
-    // (a 16-column tile stays with the first)
+    // EPI = 8: warps ew and ew + 4 share a quadrant and split its columns in
+    // whole 16-column chunks (a 16-column tile stays with the first)
     const int ew = warp - 2;
-    const bool split_cols = EPI == 8 && p.BN >= 32;
-    const int c_begin = split_cols ? (ew >> 2) * (p.BN / 2) : 0;
-    const bool idle = EPI == 8 && !split_cols && ew >= 4;
-    const int c_end = idle ? 0 : (split_cols ? c_begin + p.BN / 2 : p.BN);
+    const int c_mid = EPI == 8 ? (p.BN / 16 + 1) / 2 * 16 : p.BN;
+    const int c_begin = ew < 4 ? 0 : c_mid;
+    const int c_end = ew < 4 ? c_mid : p.BN;
+    const bool idle = c_begin >= c_end;
     const int dv = p.sh.dv_out, dh = p.sh.dh_out;
     const uint32_t M = (uint32_t)p.sh.M;
     const int64_t P = p.sh.P;
@@ -1131,13 +1131,13 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
   if (KS > kb_count) KS = kb_count;
   const int CS = (sh.csep && np == 2) ? 1 : 0;
   const int NA = KS + CS;
-  // BN: the widest tile whose NA accumulators fit TMEM (double-buffered when
-  // they fit twice)
-  int BN = Nr >= 256 ? 256 : Nr;
-  while (BN > 16 && NA * BN > 512) BN /= 2;
-  // a short K (at most 16 k-chunks) needs the epilogue overlap of two buffers
-  if (kb_count <= 16)
-    while (BN > 16 && 2 * NA * BN > 512) BN /= 2;
+  // BN: the widest tile that divides Nr in whole 16-column chunks and whose NA
+  // accumulators fit TMEM (twice where K is short, at most 16 k-chunks, which
+  // needs the epilogue overlap of two buffers)
+  const int cols_max = 512 / (kb_count <= 16 ? 2 * NA : NA);
+  int BN = Nr < 256 ? Nr : 256;
+  if (BN > cols_max) BN = cols_max / 16 * 16;
+  while (BN > 16 && Nr % BN != 0) BN -= 16;
   const int tiles_m = (int)((sh.M + BM - 1) / BM);
   // The 2-SM UMMA when the 128-row tiles pair up and each CTA's half of the
   // Bt tile is a whole number of 8-row swizzle groups.

@@ -1,14 +1,16 @@
 """The tensor-core step's tiles and stores (rows taken m_hi first, 32-byte
 stores, items loaded 32 at a time) against the oracles, at the shapes where
 they change: P below, at and above a tile's rows, runs of 1 to 16 entries,
-batches, ragged lane counts around 32 items, and a workspace that is aligned to 16 bytes only.  Tolerance: 1e-5 normwise
+batches, ragged lane counts around 32 items, bonds that are not powers of two,
+and a workspace that is aligned to 16 bytes only.  Tolerance: 1e-5 normwise
 (FP16X3), as for every other path of that form."""
 import numpy as np
 import pytest
 
 from oracle import peps as op
+from oracle import statevector as sv
 from paper_1905_08394_gb300 import binding as B
-from rqc_inputs import make_circuit, uniform_bitstrings
+from rqc_inputs import make_circuit, make_circuit_general, uniform_bitstrings
 
 pytestmark = pytest.mark.gpu
 
@@ -36,6 +38,20 @@ def test_steps_on_the_tensor_cores(cuda_device, R, C, d, n, kw):
     sim = Simulator(R, C, device=cuda_device.index or 0)
     sim.apply_circuit(circ)
     out = sim.amplitudes(bits, precision="fp16x3", flags=B.PEPS_FLAG_STEPWISE, **kw)
+    assert sim.stats()["launches_contract_tc"] > 0
+    assert relerr(out, ref) < TOL
+    sim.close()
+
+
+def test_bonds_that_are_not_powers_of_two(cuda_device):
+    from paper_1905_08394_gb300 import Simulator
+
+    circ = make_circuit_general(4, 5, 5, 7)
+    bits = uniform_bitstrings(20, 35, 7)
+    ref = sv.amplitudes(20, circ.gates, bits)
+    sim = Simulator(4, 5, device=cuda_device.index or 0)
+    sim.apply_circuit(circ)
+    out = sim.amplitudes(bits, precision="fp16x3", max_lanes=35)
     assert sim.stats()["launches_contract_tc"] > 0
     assert relerr(out, ref) < TOL
     sim.close()
