@@ -2495,7 +2495,8 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
           S.contract_tc_flops += l.flops;
           S.contract_tc_bytes += l.bytes;
         } else {
-          CUDA_TRY(launch_contract_simt(l.shape, items + l.items_off, l.n_items, ops, recs, st, s));
+          CUDA_TRY(launch_contract_simt(l.shape, items + l.items_off, l.n_items, ops, recs, st, s,
+                                        (uintptr_t)base % 32 == 0));
         }
         if (timing) {
           CUDA_TRY(record(c->ev[2 * *n_timed + 1]));

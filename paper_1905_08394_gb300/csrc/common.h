@@ -331,7 +331,7 @@ cudaError_t launch_build_tc_operands(int n_ops, int64_t max_kn, OpDesc *d_ops, i
                                      cudaStream_t s);
 cudaError_t launch_contract_simt(const StepShape &sh, const StepItem *d_items, int n_items,
                                  const OpDesc *d_ops, Rec *d_recs, const DeviceStatus *st,
-                                 cudaStream_t s);
+                                 cudaStream_t s, bool aligned32);
 // Whole sweeps of small lattices in one persistent launch (contract_small.cu):
 // the plan's steps and their first operand index, the bitstrings and the
 // FP64 amplitude accumulators; cap_g / cap_e = entries of the largest running

@@ -67,27 +67,6 @@ template <> struct FormTraits<FMT_BF16X2> { static constexpr int NP = 2, ESZ = 2
 template <> struct FormTraits<FMT_FP16X2> { static constexpr int NP = 2, ESZ = 2, KIND = 0, AB = 0; };
 template <> struct FormTraits<FMT_TF32>   { static constexpr int NP = 1, ESZ = 4, KIND = 1, AB = 2; };
 
-// x / d and x % d for a divisor fixed per launch (1 <= d <= 2^31, 0 <= x <
-// 2^31), branch-free: q = (mulhi(m, x) + x) >> l with l = ceil(log2 d) and
-// m = floor(2^32 (2^l - d) / d) + 1 (Granlund and Montgomery, "Division by
-// invariant integers using multiplication", 1994).  One form for every
-// divisor: a branch between a shift and a 64-bit division put the division's
-// code between the hot instructions, and the tile set-up alone took about
-// 1700 of a 128 x 128 tile's 6200 cycles.
-struct Div {
-  uint32_t d, m;
-  int32_t l;
-  int32_t pad_;
-  __device__ __forceinline__ uint32_t q(uint32_t x) const { return (__umulhi(m, x) + x) >> l; }
-  __device__ __forceinline__ uint32_t r(uint32_t x) const { return x - q(x) * d; }
-};
-inline Div make_div(int64_t d) {
-  Div v{(uint32_t)(d > 0 ? d : 1), 0u, 0, 0};
-  while (((int64_t)1 << v.l) < (int64_t)v.d) ++v.l;
-  v.m = (uint32_t)(((((uint64_t)1 << v.l) - v.d) << 32) / v.d + 1);
-  return v;
-}
-
 struct __align__(128) TcParams {   // the tensor maps need 128-byte alignment
   CUtensorMap mapA;        // {k, m, plane, lane}; m_hi-major steps: {k, m_hi, m_lo, b, plane/lane}
   CUtensorMap mapB[2];     // [plane] {k, n, operand variant}

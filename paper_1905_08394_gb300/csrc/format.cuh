@@ -10,6 +10,27 @@
 
 namespace peps {
 
+// x / d and x % d for a divisor fixed per launch (1 <= d <= 2^31, 0 <= x <
+// 2^31), branch-free: q = (mulhi(m, x) + x) >> l with l = ceil(log2 d) and
+// m = floor(2^32 (2^l - d) / d) + 1 (Granlund and Montgomery, "Division by
+// invariant integers using multiplication", 1994).  One form for every
+// divisor: with a branch between a shift and a 64-bit division the division's
+// code lies between the hot instructions, and the tensor-core kernel's tile
+// set-up alone took about 1700 of a 128 x 128 tile's 6200 cycles.
+struct Div {
+  uint32_t d, m;
+  int32_t l;
+  int32_t pad_;
+  __device__ __forceinline__ uint32_t q(uint32_t x) const { return (__umulhi(m, x) + x) >> l; }
+  __device__ __forceinline__ uint32_t r(uint32_t x) const { return x - q(x) * d; }
+};
+inline Div make_div(int64_t d) {
+  Div v{(uint32_t)(d > 0 ? d : 1), 0u, 0, 0};
+  while (((int64_t)1 << v.l) < (int64_t)v.d) ++v.l;
+  v.m = (uint32_t)(((((uint64_t)1 << v.l) - v.d) << 32) / v.d + 1);
+  return v;
+}
+
 __device__ __forceinline__ float round_tf32(float x) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
@@ -105,68 +126,8 @@ __device__ __forceinline__ float2 store_g(void *base, int64_t e, int64_t plane, 
   }
 }
 
-// Store 8 consecutive complex entries dest0 .. dest0+7 (dest0 % 8 == 0) from
-// 16 floats (re, im interleaved) scaled by 2^x, with 16-byte vector stores.
-// Returns the max |stored component|.
 // 2^x as a float, x in [-126, 127] (exact).
 __device__ __forceinline__ float pow2f(int x) { return __int_as_float((127 + x) << 23); }
-
-// Store 8 consecutive complex entries dest0 .. dest0+7 (dest0 % 8 == 0) from
-// 16 floats (re, im interleaved) multiplied by sc (a power of two), with
-// 16-byte vector stores.  Returns the max |scaled component| before rounding
-// to the storage format (step_scale_exp allows for the rounding).
-template <int FMT>
-__device__ __forceinline__ float store8_g(void *base, int64_t dest0, int64_t plane,
-                                          const float (&v)[16], float sc) {
-  float m = 0.f;
-  float o[16];
-#pragma unroll
-  for (int i = 0; i < 16; ++i) {
-    o[i] = v[i] * sc;
-    m = fmaxf(m, fabsf(o[i]));
-  }
-  if (FMT == FMT_F32 || FMT == FMT_TF32) {
-    if (FMT == FMT_TF32) {
-#pragma unroll
-      for (int i = 0; i < 16; ++i) o[i] = round_tf32(o[i]);
-    }
-    uint4 *d = reinterpret_cast<uint4 *>(reinterpret_cast<float2 *>(base) + dest0);
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-      d[i] = make_uint4(__float_as_uint(o[4 * i]), __float_as_uint(o[4 * i + 1]),
-                        __float_as_uint(o[4 * i + 2]), __float_as_uint(o[4 * i + 3]));
-  } else if (FMT == FMT_BF16 || FMT == FMT_FP16) {
-    uint32_t w[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j)
-      w[j] = FMT == FMT_BF16 ? pack_bf16(o[2 * j], o[2 * j + 1]) : pack_f16(o[2 * j], o[2 * j + 1]);
-    uint4 *d = reinterpret_cast<uint4 *>(reinterpret_cast<uint32_t *>(base) + dest0);
-    d[0] = make_uint4(w[0], w[1], w[2], w[3]);
-    d[1] = make_uint4(w[4], w[5], w[6], w[7]);
-  } else {
-    uint32_t hi[8], lo[8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      if (FMT == FMT_BF16X2) {
-        hi[j] = pack_bf16(o[2 * j], o[2 * j + 1]);
-        const float2 h = unpack_bf16(hi[j]);
-        lo[j] = pack_bf16(o[2 * j] - h.x, o[2 * j + 1] - h.y);
-      } else {
-        hi[j] = pack_f16(o[2 * j], o[2 * j + 1]);
-        const float2 h = unpack_f16(hi[j]);
-        lo[j] = pack_f16(o[2 * j] - h.x, o[2 * j + 1] - h.y);
-      }
-    }
-    uint32_t *p = reinterpret_cast<uint32_t *>(base);
-    uint4 *dh = reinterpret_cast<uint4 *>(p + dest0);
-    uint4 *dl = reinterpret_cast<uint4 *>(p + plane / 2 + dest0);
-    dh[0] = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-    dh[1] = make_uint4(hi[4], hi[5], hi[6], hi[7]);
-    dl[0] = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-    dl[1] = make_uint4(lo[4], lo[5], lo[6], lo[7]);
-  }
-  return m;
-}
 
 // 8 complex entries (16 floats, re / im interleaved) in a storage format:
 // F32 / TF32 two words per entry; BF16 / FP16 one word (re, im) per entry;
