@@ -58,7 +58,16 @@ constexpr int BM = 128;
 // Warps: a TMA producer, an MMA issuer and EPI epilogue warps; EPI = 4 (one per
 // TMEM lane quadrant) or 8 (two per quadrant, each draining half of the
 // tile's columns, for steps whose epilogue outlasts their MMAs).
-constexpr int threads_of(int epi) { return 64 + 32 * epi; }
+// DR = 1 (a draining epilogue, eight warps): the accumulators take all of TMEM
+// (256 columns of main and of correction sums), so a tile's MMAs wait for the
+// epilogue of the one before.  A warp then reads its 128 columns into registers
+// at once (the two sums added), releases TMEM, and scales, splits and stores
+// from registers under the next tile's MMAs.  Its 128 held values need more
+// registers than a thread gets at launch, so the producer's warpgroup (the
+// producer, the MMA issuer and two idle warps) gives some up: 384 threads x 168
+// = 128 x 72 + 256 x 216.
+constexpr int first_epi(int dr) { return dr ? 4 : 2; }
+constexpr int threads_of(int epi, int dr) { return 32 * (first_epi(dr) + epi); }
 
 template <int FMT> struct FormTraits;
 template <> struct FormTraits<FMT_BF16>   { static constexpr int NP = 1, ESZ = 2, KIND = 0, AB = 1; };
@@ -98,9 +107,8 @@ struct __align__(128) TcParams {   // the tensor maps need 128-byte alignment
   int64_t mlo;  // m_hi-major: Mr / P
   int64_t watchdog_ns;
   double2 *dot_partials;   // sh.dot: [item][tiles_per_item * CG * EPI]
-  int blocked;  // 1: CTA pair c takes the consecutive tiles [c per, (c + 1) per)
-                // (an item's tiles in a row, so its variant, scale and
-                // addresses are set up once); 0: tiles c, c + pairs, ...
+  int blocked;  // 1: CTA pair c takes the consecutive tiles [c per, (c + 1) per);
+                // 0: tiles c, c + pairs, ...
   // divisors of the tile and store index arithmetic
   Div d_tpi, d_tn;             // tiles per item, column tiles
   Div d_hper, d_lper, d_ph, d_lh;  // m_hi-major tiles: P / ph, (Mr / P) / lh, ph, lh
@@ -169,7 +177,7 @@ struct Watch {
 __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, Watch &w) {
   uint32_t spins = 0;
   while (!mbar_test(bar, parity)) {
-    if ((++spins & 63) == 0) {
+    if ((++spins & 63) == 8) {   // on the eighth failed try, then on every 64th
       if (*w.abort) return false;
       if (globaltimer() > w.deadline) {
         *w.abort = 1;
@@ -185,9 +193,9 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, Watch 
 }
 
 // What the producer and the epilogue need of the launch's items, one item per
-// lane: the tiles of a CTA pair run through consecutive items (the item index
-// grows by 0 or 1 from tile to tile), so a warp loads the next 32 items'
-// entries at once and takes an item's from its lane by a shuffle.  Loaded one
+// lane: the tiles of a CTA pair run through the items in increasing order, so a
+// warp loads the next 32 items' entries at once and takes an item's from its
+// lane by a shuffle.  Loaded one
 // by one, the chain item -> bitstring -> operand -> record costs three
 // dependent misses per item, which bounds launches of a tile or two per item.
 struct ItemBlock {
@@ -393,8 +401,8 @@ __device__ __forceinline__ void tmem_wait2(uint32_t (&r)[16], uint32_t (&q)[16])
 // ---------------------------------------------------------------------------
 // CG: CTAs per MMA.  CG = 1: one CTA per 128-row tile.  CG = 2: a cluster of
 // two CTAs per 256-row tile (2-SM UMMA), see the file comment.
-template <int FMT, int ROWB, int CG, int EPI>
-__global__ void __launch_bounds__(threads_of(EPI), 1)
+template <int FMT, int ROWB, int CG, int EPI, int DR>
+__global__ void __launch_bounds__(threads_of(EPI, DR), 1)
     k_contract_tc(const __grid_constant__ TcParams p) {
   using T = FormTraits<FMT>;
   constexpr int NP = T::NP;
@@ -474,6 +482,9 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
   const uint32_t full0 = CG == 2 ? cluster_addr(full, 0) : 0u;
   const uint32_t tempty0 = CG == 2 ? cluster_addr(tempty, 0) : 0u;
 
+  if (warp < first_epi(DR)) {
+  // DR: the warpgroups' register shares, 72 x 128 + 216 x 256 = 168 x 384
+  if constexpr (DR != 0) asm volatile("setmaxnreg.dec.sync.aligned.u32 72;");
   if (warp == 0) {
     // ---------------- TMA producer (both CTAs) ----------------
     uint32_t it = 0;
@@ -643,8 +654,10 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
       w2.abort = &zero;
       mbar_wait(done, 0u, w2);
     }
+  }
   } else {
     // ---------------- epilogue (both CTAs) ----------------
+    if constexpr (DR != 0) asm volatile("setmaxnreg.inc.sync.aligned.u32 216;");
     // Warp w drains TMEM lanes 32*(w%4) .. +31 (the rows it may access), all
     // columns of the tile, 16 at a time; the load of chunk c+1 is in flight
     // while chunk c is scaled, split and stored.
@@ -652,7 +665,7 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
     const int row = 32 * quad + lane;
     // EPI = 8: warps ew and ew + 4 share a quadrant and split its columns in
     // whole 16-column chunks (a 16-column tile stays with the first)
-    const int ew = warp - 2;
+    const int ew = warp - first_epi(DR);
     const int c_mid = EPI == 8 ? (p.BN / 16 + 1) / 2 * 16 : p.BN;
     const int c_begin = ew < 4 ? 0 : c_mid;
     const int c_end = ew < 4 ? c_mid : p.BN;
@@ -761,9 +774,86 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
       const uint32_t tbase =
           tmem_base + ((uint32_t)(32 * quad) << 16) + (uint32_t)(acc * BN * KSP);
       float dre = 0.f, dim = 0.f;   // fused dot: this row's partial sum
-      // The columns in chunks of 16 (8 complex entries), the next chunk (or
-      // pair) loaded from TMEM while the current one is used.
+      // TMEM read: the accumulator goes back to the MMA issuer
+      auto release = [&]() {
+        tc_fence_before();
+        if (CG == 1) {
+          mbar_arrive(&tempty[acc]);
+        } else {
+          __syncwarp();
+          if (lane == 0) mbar_arrive_cluster(tempty0 + (uint32_t)acc * 8u);
+        }
+      };
+      // The columns in chunks of 16 (8 complex entries), the next chunk loaded
+      // from TMEM while the current one is used.
       uint32_t ra[16], rb[16];
+      if constexpr (DR != 0) {
+        // this warp's 128 columns (BN = 256) into registers
+        uint32_t v[8][16];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) tmem_ld16_issue(tbase + (uint32_t)(c_begin + 16 * j), v[j]);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) tmem_wait(v[j]);
+        for (int sg = 1; sg < KSP; ++sg) {
+          const uint32_t cb = tbase + (uint32_t)(sg * BN + c_begin);
+          tmem_ld16_issue(cb, ra);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            uint32_t (&cur)[16] = j & 1 ? rb : ra, (&next)[16] = j & 1 ? ra : rb;
+            tmem_wait(cur);
+            if (j < 7) tmem_ld16_issue(cb + (uint32_t)(16 * (j + 1)), next);
+#pragma unroll
+            for (int i = 0; i < 16; ++i)
+              v[j][i] = __float_as_uint(__uint_as_float(v[j][i]) + __uint_as_float(cur[i]));
+          }
+        }
+        release();
+        if (dotm) {
+          const int64_t dot_e = (int64_t)m_lo * p.sh.N + ((nt * BN + c_begin) >> 1);
+          if (live) {
+            Raw8 fcur, fnext;
+            load8_raw<FMT>(D, dot_e, p.sh.plane, fcur);
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              if (j < 7) load8_raw<FMT>(D, dot_e + 8 * (j + 1), p.sh.plane, fnext);
+              float2 f[8];
+              unpack8<FMT>(fcur, f);
+#pragma unroll
+              for (int q = 0; q < 8; ++q) {
+                const float vr = __uint_as_float(v[j][2 * q]), vi = __uint_as_float(v[j][2 * q + 1]);
+                dre = fmaf(vr, f[q].x, fmaf(-vi, f[q].y, dre));
+                dim = fmaf(vr, f[q].y, fmaf(vi, f[q].x, dim));
+              }
+              fcur = fnext;
+            }
+          }
+        } else {
+          // runs of 8 entries (the rule that takes this form)
+          const int64_t base = !vbm ? (int64_t)b * MrN + ((int64_t)m_lo * dh * P + m_hi) * dv
+                                    : (int64_t)b * dv * Mrdh + (int64_t)m_lo * dh * P + m_hi;
+          const uint32_t nc0 = (uint32_t)(nt * BN + c_begin) >> 1;
+          const uint32_t cq = flat ? 0u : dR.q(nc0);
+          uint32_t cr = flat ? nc0 : nc0 - cq * R;
+          int64_t dest = base + (int64_t)cq * stride_q + (int64_t)cr;
+          if (live) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+              float o[16];
+#pragma unroll
+              for (int i = 0; i < 16; ++i) o[i] = __uint_as_float(v[j][i]);
+              Packed8<FMT> w;
+              vmax = fmaxf(vmax, pack8<FMT>(o, sc, w));
+              store_run8_wide<FMT>(D, dest, p.sh.plane, w);
+              cr += 8;
+              dest += 8;
+              if (cr == R) {
+                cr = 0;
+                dest += wrap;
+              }
+            }
+          }
+        }
+      } else {
       if (!idle) tmem_ld16_issue(tbase + (uint32_t)c_begin, ra);
       if (dotm) {
         // fused dot: the partner entries of row m (P = 1, row-major m N + n),
@@ -815,15 +905,11 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
             dest += wrap;
           }
         };
-        // the next 16 accumulator columns (8 complex entries): scaled, rounded
-        // to the storage format and stored in runs of W
-        auto emit = [&](const float (&o)[16]) {
-          Packed8<FMT> w;
-          vmax = fmaxf(vmax, pack8<FMT>(o, sc, w));
+        // the next 8 entries in runs of W
+        auto store_any = [&](const Packed8<FMT> &w) {
           switch (W) {
             case 8:
-              if (p.wide) store_run8_wide<FMT>(D, dest, p.sh.plane, w);
-              else store_run<FMT, 8>(D, dest, p.sh.plane, w, 0);
+              store_run<FMT, 8>(D, dest, p.sh.plane, w, 0);
               advance(8);
               break;
             case 4:
@@ -848,66 +934,82 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
               }
           }
         };
-        // the other K segments of chunk c, added with FP32 round-to-nearest
-        auto add_segments = [&](int c, float (&o)[16]) {
-          for (int sg = 1; sg < KSP; ++sg) {
-            uint32_t rc[16];
-            tmem_ld16_issue(tbase + (uint32_t)(sg * BN + c), rc);
-            tmem_wait(rc);
-#pragma unroll
-            for (int i = 0; i < 16; ++i) o[i] += __uint_as_float(rc[i]);
-          }
-        };
-        if (EPI == 4) {
-          // two chunks per iteration (twice the independent work in flight);
-          // the next pair's TMEM loads overlap this pair's arithmetic
-          if (c_begin + 16 < c_end) tmem_ld16_issue(tbase + (uint32_t)(c_begin + 16), rb);
+        // 16 accumulator columns (8 complex entries) at a time: the other
+        // accumulators added with FP32 round-to-nearest, scaled, rounded to the
+        // storage format and stored, while the next chunk (of the first two
+        // accumulators) is loaded.  One loop for the usual runs of 8, with no
+        // choice between a chunk's load and its store, and one for the rest.
+        auto chunks = [&](auto store) {
+          const bool pair = KSP > 1;
+          const uint32_t t2 = tbase + (uint32_t)BN;
+          if (pair && !idle) tmem_ld16_issue(t2 + (uint32_t)c_begin, rb);
           tmem_wait2(ra, rb);
-          for (int c = c_begin; c < c_end; c += 32) {
-            const bool two = c + 16 < c_end;
-            float o0[16], o1[16];
-#pragma unroll
-            for (int i = 0; i < 16; ++i) {
-              o0[i] = __uint_as_float(ra[i]);
-              o1[i] = __uint_as_float(rb[i]);
-            }
-            const bool more = c + 32 < c_end;
-            if (more) {
-              tmem_ld16_issue(tbase + (uint32_t)(c + 32), ra);
-              if (c + 48 < c_end) tmem_ld16_issue(tbase + (uint32_t)(c + 48), rb);
-            }
-            add_segments(c, o0);
-            if (two) add_segments(c + 16, o1);
-            if (live) {
-              emit(o0);
-              if (two) emit(o1);
-            }
-            if (more) tmem_wait2(ra, rb);
-          }
-        } else {
-          // one chunk at a time (the register budget of eight epilogue warps),
-          // one copy of the code in the loop (the instruction cache holds the
-          // three roles' loops at once): chunk c is copied out of the load
-          // registers, chunk c + 16 loads into them while c is used
-          tmem_wait(ra);
           for (int c = c_begin; c < c_end; c += 16) {
             const bool more = c + 16 < c_end;
             float o[16];
 #pragma unroll
             for (int i = 0; i < 16; ++i) o[i] = __uint_as_float(ra[i]);
-            if (more) tmem_ld16_issue(tbase + (uint32_t)(c + 16), ra);
-            add_segments(c, o);
-            if (live) emit(o);
-            if (more) tmem_wait(ra);
+            if (pair) {
+#pragma unroll
+              for (int i = 0; i < 16; ++i) o[i] += __uint_as_float(rb[i]);
+            }
+            if (more) {
+              tmem_ld16_issue(tbase + (uint32_t)(c + 16), ra);
+              if (pair) tmem_ld16_issue(t2 + (uint32_t)(c + 16), rb);
+            }
+            for (int sg = 2; sg < KSP; ++sg) {
+              uint32_t rc[16];
+              tmem_ld16_issue(tbase + (uint32_t)(sg * BN + c), rc);
+              tmem_wait(rc);
+#pragma unroll
+              for (int i = 0; i < 16; ++i) o[i] += __uint_as_float(rc[i]);
+            }
+            if (live) {
+              Packed8<FMT> w;
+              vmax = fmaxf(vmax, pack8<FMT>(o, sc, w));
+              store(w);
+            }
+            if (more) tmem_wait2(ra, rb);
           }
+        };
+        auto store8 = [&](const Packed8<FMT> &w) {
+          store_run8_wide<FMT>(D, dest, p.sh.plane, w);
+          advance(8);
+        };
+        if (W == 8 && p.wide) {
+          if (NP == 1 && KSP == 1) {
+            // single-plane forms: less arithmetic per chunk, so the chunk is
+            // used where it was loaded, the two buffers in turn (16 lanes of
+            // 32768 x 64 x 64 in BF16: 52.6 -> 47.7 us)
+            auto emit = [&](const uint32_t (&r)[16]) {
+              if (!live) return;
+              float o[16];
+#pragma unroll
+              for (int i = 0; i < 16; ++i) o[i] = __uint_as_float(r[i]);
+              Packed8<FMT> w;
+              vmax = fmaxf(vmax, pack8<FMT>(o, sc, w));
+              store8(w);
+            };
+            tmem_wait(ra);
+            for (int c = c_begin; c < c_end; c += 32) {
+              const bool two = c + 16 < c_end, more = c + 32 < c_end;
+              if (two) tmem_ld16_issue(tbase + (uint32_t)(c + 16), rb);
+              emit(ra);
+              if (two) {
+                tmem_wait(rb);
+                if (more) tmem_ld16_issue(tbase + (uint32_t)(c + 32), ra);
+                emit(rb);
+                if (more) tmem_wait(ra);
+              }
+            }
+          } else {
+            chunks(store8);
+          }
+        } else {
+          chunks(store_any);
         }
       }
-      tc_fence_before();
-      if (CG == 1) {
-        mbar_arrive(&tempty[acc]);
-      } else {
-        __syncwarp();
-        if (lane == 0) mbar_arrive_cluster(tempty0 + (uint32_t)acc * 8u);
+      release();
       }
       if (dotm) {
         // the warp's 32 rows summed in FP64, one slot per (tile, CTA, warp)
@@ -920,7 +1022,7 @@ __global__ void __launch_bounds__(threads_of(EPI), 1)
           p.dot_partials[((int64_t)item * tiles_per_item + rem) * (CG * EPI) + (int)rank * EPI +
                          ew] = make_double2(r, i);
       }
-      if (mt == 0 && nt == 0 && warp == 2 && lane == 0) p.recs[out_rec].exp = out_exp;
+      if (mt == 0 && nt == 0 && ew == 0 && lane == 0) p.recs[out_rec].exp = out_exp;
     }
     if (!dotm && cached_item >= 0) flush_max();
   }
@@ -1005,6 +1107,7 @@ struct TcLaunchData {
   int rowb;
   int cg;   // CTAs per MMA: 1, or 2 for the 2-SM UMMA
   int epi;  // epilogue warps: 4, or 8 where the epilogue bounds the step
+  int dr;   // 1: the draining epilogue
 };
 
 int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
@@ -1117,6 +1220,22 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
   int BN = Nr < 256 ? Nr : 256;
   if (BN > cols_max) BN = cols_max / 16 * 16;
   while (BN > 16 && Nr % BN != 0) BN -= 16;
+  // entries in contiguous runs of 8 (the epilogue's W = 8)
+  const int run = sh.vb && sh.nvs ? sh.dh_out : (sh.dv_out == 1 && sh.P == 1 ? sh.N : sh.dv_out);
+  const bool runs8 = !sh.dot && run % 8 == 0 && (sh.vb ? sh.nvs && sh.P == 1 : true);
+  // The draining epilogue where main and correction accumulators fill TMEM on
+  // 256-column tiles.  For a short K that is the alternative to 128-column
+  // tiles with two buffers, which load every row of A twice as often: 16 lanes
+  // of 65536 x 256 x 256 took 1408 us that way, at 9 TB/s from L2 into shared
+  // memory; 1072 us now (512 lanes of the fused 1024 x 1024 x 256 merge: 1912 ->
+  // 1756 us).  It needs tiles for every CTA pair; the fused dot's
+  // tiles keep their width (it fixes the order of its partial sums).
+  const bool wide32 = (uintptr_t)a_base % 32 == 0;
+  const bool drain =
+      CS == 1 && NA == 2 && rowb == 128 && Nr % 256 == 0 && epi != 4 && wide32 &&
+      (sh.dot ? BN == 256
+              : runs8 && (BN == 256 || (sh.M / 256) * (Nr / 256) * (int64_t)a_lanes >= 152));
+  if (drain) BN = 256;
   const int tiles_m = (int)((sh.M + BM - 1) / BM);
   // The 2-SM UMMA when the 128-row tiles pair up and each CTA's half of the
   // Bt tile is a whole number of 8-row swizzle groups.
@@ -1143,7 +1262,7 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
     }
   }
   d->prm.sh = sh;
-  d->prm.wide = ((uintptr_t)a_base % 32 == 0) ? 1 : 0;
+  d->prm.wide = wide32 ? 1 : 0;
   d->prm.BN = BN;
   d->prm.tiles_m = (int)((sh.M + BM - 1) / BM);
   d->prm.tiles_n = Nr / BN;
@@ -1153,8 +1272,17 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
   {
     const int mgroups = d->prm.tiles_m / d->cg;
     d->prm.gm = (d->prm.tiles_n >= 32 && mgroups >= 16) ? 8 : 1;
-    // outside the grouped order a pair walks consecutive tiles
-    d->prm.blocked = d->prm.gm == 1 ? 1 : 0;
+    // Outside the grouped order a pair walks consecutive tiles (an item's
+    // set-up and operand once), or every ncl-th where the tiles are long and a
+    // row panel has several of them: the pairs then work on the same k-slabs of
+    // A and B at the same time, which L2 serves once, while consecutive tiles
+    // re-read a panel of A after it has left.  Consecutive / interleaved: 32 lanes
+    // of 512 x 1024 x 1024 339 / 226 us, 16 of 65536 x 256 x 256 1072 / 998 us,
+    // 512 of 4096 x 64 x 256 908 / 846 us; but 512 of 2048 x 16 x 64 117 / 145 us,
+    // 16 of 4096 x 64 x 512 60.2 / 61.8 us.
+    const bool interleave = d->prm.tiles_n >= 2 && BN == 256 &&
+                            (sh.K >= 128 || (sh.K >= 64 && d->prm.tiles_n == 2));
+    d->prm.blocked = d->prm.gm == 1 && !interleave ? 1 : 0;
     d->prm.d_tpi = make_div((int64_t)mgroups * d->prm.tiles_n);
     d->prm.d_tn = make_div(d->prm.tiles_n);
   }
@@ -1194,22 +1322,24 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
   const bool epi_bound = sh.dot || d->prm.nbuf == 1 || (sh.K <= 64 && BN >= 64) ||
                          (sh.K <= 32 && BN >= 32);
   d->epi = epi == 4 || epi == 8 ? epi : (epi_bound ? 8 : 4);
+  d->dr = drain ? 1 : 0;
+  if (drain) d->epi = 8;
   *out_handle = d;
   return stages >= 2 ? 0 : -5;
 }
 
 void tc_release(void *h) { delete (TcLaunchData *)h; }
 
-template <int FMT, int ROWB, int CG, int EPI>
+template <int FMT, int ROWB, int CG, int EPI, int DR>
 static int &max_clusters_of() {
   static int v = -1;  // co-resident clusters at the largest smem size (-1: not set up)
   return v;
 }
 
-template <int FMT, int ROWB, int CG, int EPI>
+template <int FMT, int ROWB, int CG, int EPI, int DR>
 static cudaError_t init_kernel() {
-  auto kern = k_contract_tc<FMT, ROWB, CG, EPI>;
-  int &max_clusters = max_clusters_of<FMT, ROWB, CG, EPI>();
+  auto kern = k_contract_tc<FMT, ROWB, CG, EPI, DR>;
+  int &max_clusters = max_clusters_of<FMT, ROWB, CG, EPI, DR>();
   if (max_clusters < 0) {
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          227 * 1024);
@@ -1221,7 +1351,7 @@ static cudaError_t init_kernel() {
     qa[0].val.clusterDim.y = 1;
     qa[0].val.clusterDim.z = 1;
     q.gridDim = dim3(CG * 64);
-    q.blockDim = dim3(threads_of(EPI));
+    q.blockDim = dim3(threads_of(EPI, DR));
     q.dynamicSmemBytes = 227 * 1024;
     q.attrs = qa;
     q.numAttrs = 1;
@@ -1236,12 +1366,12 @@ static cudaError_t init_kernel() {
   return cudaSuccess;
 }
 
-template <int FMT, int ROWB, int CG, int EPI>
+template <int FMT, int ROWB, int CG, int EPI, int DR>
 static cudaError_t launch_one(const TcParams &prm, int units, size_t smem, cudaStream_t s) {
-  auto kern = k_contract_tc<FMT, ROWB, CG, EPI>;
-  cudaError_t e0 = init_kernel<FMT, ROWB, CG, EPI>();
+  auto kern = k_contract_tc<FMT, ROWB, CG, EPI, DR>;
+  cudaError_t e0 = init_kernel<FMT, ROWB, CG, EPI, DR>();
   if (e0 != cudaSuccess) return e0;
-  const int max_clusters = max_clusters_of<FMT, ROWB, CG, EPI>();
+  const int max_clusters = max_clusters_of<FMT, ROWB, CG, EPI, DR>();
   // units = SMs to use; one CTA per SM, clusters of CG
   int clusters = units / CG;
   if (max_clusters > 0 && clusters > max_clusters) clusters = max_clusters;
@@ -1253,7 +1383,7 @@ static cudaError_t launch_one(const TcParams &prm, int units, size_t smem, cudaS
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   cfg.gridDim = dim3(clusters * CG);
-  cfg.blockDim = dim3(threads_of(EPI));
+  cfg.blockDim = dim3(threads_of(EPI, DR));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = attr;
@@ -1261,43 +1391,49 @@ static cudaError_t launch_one(const TcParams &prm, int units, size_t smem, cudaS
   return cudaLaunchKernelEx(&cfg, kern, prm);
 }
 
-template <int FMT, int EPI>
-static cudaError_t warm_epi(int rowb, int cg) {
-  if (rowb == 128)
-    return cg == 2 ? init_kernel<FMT, 128, 2, EPI>() : init_kernel<FMT, 128, 1, EPI>();
-  return cg == 2 ? init_kernel<FMT, 64, 2, EPI>() : init_kernel<FMT, 64, 1, EPI>();
+// f.run<FMT, ROWB, CG, EPI, DR>() for the kernel that `d` launches
+// (the draining form exists for the split formats and 128-byte stages only).
+template <int FMT, class F>
+static cudaError_t with_kernel(const TcLaunchData *d, F f) {
+  if constexpr (FormTraits<FMT>::NP == 2) {
+    if (d->dr) return d->cg == 2 ? f.template run<FMT, 128, 2, 8, 1>() : f.template run<FMT, 128, 1, 8, 1>();
+  }
+  if (d->dr) return cudaErrorInvalidValue;
+  if (d->epi == 8) {
+    if (d->rowb == 128)
+      return d->cg == 2 ? f.template run<FMT, 128, 2, 8, 0>() : f.template run<FMT, 128, 1, 8, 0>();
+    return d->cg == 2 ? f.template run<FMT, 64, 2, 8, 0>() : f.template run<FMT, 64, 1, 8, 0>();
+  }
+  if (d->rowb == 128)
+    return d->cg == 2 ? f.template run<FMT, 128, 2, 4, 0>() : f.template run<FMT, 128, 1, 4, 0>();
+  return d->cg == 2 ? f.template run<FMT, 64, 2, 4, 0>() : f.template run<FMT, 64, 1, 4, 0>();
 }
-template <int FMT>
-static cudaError_t warm_fmt(int rowb, int cg, int epi) {
-  return epi == 8 ? warm_epi<FMT, 8>(rowb, cg) : warm_epi<FMT, 4>(rowb, cg);
-}
-
-cudaError_t tc_warm(void *handle) {
-  TcLaunchData *d = (TcLaunchData *)handle;
+template <class F>
+static cudaError_t with_kernel_of(const TcLaunchData *d, F f) {
   switch (d->prm.sh.fmt) {
-    case FMT_BF16: return warm_fmt<FMT_BF16>(d->rowb, d->cg, d->epi);
-    case FMT_FP16: return warm_fmt<FMT_FP16>(d->rowb, d->cg, d->epi);
-    case FMT_BF16X2: return warm_fmt<FMT_BF16X2>(d->rowb, d->cg, d->epi);
-    case FMT_FP16X2: return warm_fmt<FMT_FP16X2>(d->rowb, d->cg, d->epi);
-    case FMT_TF32: return warm_fmt<FMT_TF32>(d->rowb, d->cg, d->epi);
+    case FMT_BF16: return with_kernel<FMT_BF16>(d, f);
+    case FMT_FP16: return with_kernel<FMT_FP16>(d, f);
+    case FMT_BF16X2: return with_kernel<FMT_BF16X2>(d, f);
+    case FMT_FP16X2: return with_kernel<FMT_FP16X2>(d, f);
+    case FMT_TF32: return with_kernel<FMT_TF32>(d, f);
   }
   return cudaErrorInvalidValue;
 }
+struct WarmKernel {
+  template <int FMT, int ROWB, int CG, int EPI, int DR>
+  cudaError_t run() const { return init_kernel<FMT, ROWB, CG, EPI, DR>(); }
+};
+struct LaunchKernel {
+  const TcParams &prm;
+  int units;
+  size_t smem;
+  cudaStream_t s;
+  template <int FMT, int ROWB, int CG, int EPI, int DR>
+  cudaError_t run() const { return launch_one<FMT, ROWB, CG, EPI, DR>(prm, units, smem, s); }
+};
 
-template <int FMT, int EPI>
-static cudaError_t launch_epi(const TcParams &prm, int rowb, int cg, int units, size_t smem,
-                              cudaStream_t s) {
-  if (rowb == 128)
-    return cg == 2 ? launch_one<FMT, 128, 2, EPI>(prm, units, smem, s)
-                   : launch_one<FMT, 128, 1, EPI>(prm, units, smem, s);
-  return cg == 2 ? launch_one<FMT, 64, 2, EPI>(prm, units, smem, s)
-                 : launch_one<FMT, 64, 1, EPI>(prm, units, smem, s);
-}
-template <int FMT>
-static cudaError_t launch_fmt(const TcParams &prm, int rowb, int cg, int epi, int units,
-                              size_t smem, cudaStream_t s) {
-  return epi == 8 ? launch_epi<FMT, 8>(prm, rowb, cg, units, smem, s)
-                  : launch_epi<FMT, 4>(prm, rowb, cg, units, smem, s);
+cudaError_t tc_warm(void *handle) {
+  return with_kernel_of((const TcLaunchData *)handle, WarmKernel{});
 }
 
 int tc_dot_slots(const void *handle) {
@@ -1326,14 +1462,7 @@ cudaError_t launch_contract_tc(void *handle, const StepItem *d_items, int n_item
   const int np = np_of(prm.sh.fmt);
   const size_t smem = (size_t)prm.stages * np * (BM + prm.BN / cg) * d->rowb + 1024 +
                       (2 * prm.stages + 6) * 8 + 16;
-  switch (prm.sh.fmt) {
-    case FMT_BF16: return launch_fmt<FMT_BF16>(prm, d->rowb, cg, d->epi, units, smem, s);
-    case FMT_FP16: return launch_fmt<FMT_FP16>(prm, d->rowb, cg, d->epi, units, smem, s);
-    case FMT_BF16X2: return launch_fmt<FMT_BF16X2>(prm, d->rowb, cg, d->epi, units, smem, s);
-    case FMT_FP16X2: return launch_fmt<FMT_FP16X2>(prm, d->rowb, cg, d->epi, units, smem, s);
-    case FMT_TF32: return launch_fmt<FMT_TF32>(prm, d->rowb, cg, d->epi, units, smem, s);
-  }
-  return cudaErrorInvalidValue;
+  return with_kernel_of(d, LaunchKernel{prm, units, smem, s});
 }
 
 // ---------------------------------------------------------------------------

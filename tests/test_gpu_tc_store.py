@@ -43,6 +43,27 @@ def test_steps_on_the_tensor_cores(cuda_device, R, C, d, n, kw):
     sim.close()
 
 
+@pytest.mark.parametrize("prec,tol", [("fp16x3", TOL), ("bf16x3", 3e-5)])
+@pytest.mark.parametrize("R,C,d,n,kw", [
+    (6, 6, 24, 18, dict()),                                 # runs of 8 over h' and v'
+    (6, 6, 24, 12, dict(scheme="quadrants")),               # merges, the fused dot, open legs
+    (5, 5, 28, 5, dict(scheme="quadrants")),                # odd side, few tiles
+])
+def test_separate_corrections_with_one_accumulator_buffer(cuda_device, prec, tol, R, C, d, n, kw):
+    # tc_ksplit = -1 gives every step a correction accumulator, so wide steps
+    # take the epilogue that drains TMEM into registers
+    from paper_1905_08394_gb300 import Simulator
+
+    circ = make_circuit(R, C, d, 5)
+    bits = uniform_bitstrings(R * C, n, 5)
+    ref = op.amplitudes(op.build(R, C, circ.gates), bits)
+    sim = Simulator(R, C, device=cuda_device.index or 0)
+    sim.apply_circuit(circ)
+    out = sim.amplitudes(bits, precision=prec, tc_ksplit=-1, **kw)
+    assert relerr(out, ref) < tol
+    sim.close()
+
+
 def test_bonds_that_are_not_powers_of_two(cuda_device):
     from paper_1905_08394_gb300 import Simulator
 
