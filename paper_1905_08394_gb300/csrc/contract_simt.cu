@@ -151,8 +151,10 @@ k_contract_simt(const __grid_constant__ SimtParams p, const StepItem *__restrict
   float2 *As = reinterpret_cast<float2 *>(simt_sm);                      // [2][ROWS][LDA]
   float *Bs = reinterpret_cast<float *>(As + 2 * ROWS * LDA);            // [2][3][BK][COLS]
 
+  pdl_trigger();
   const StepItem it = items[blockIdx.z];
   const OpDesc &op = ops[it.op_base + block_variant(*it.bits, p.sh)];
+  pdl_wait();
   const float2 *__restrict__ Ec = op.Ec;
   const int64_t M = p.sh.M;
   const int K = p.sh.K, N = p.sh.N;
@@ -367,9 +369,11 @@ template <int FMT>
 __global__ void __launch_bounds__(256)
 k_contract_rows(const StepShape sh, const StepItem *__restrict__ items,
                 const OpDesc *__restrict__ ops, Rec *__restrict__ recs) {
+  pdl_trigger();
   const StepItem it = items[blockIdx.y];
   const uint64_t bits = *it.bits;
   const OpDesc &op = ops[it.op_base + block_variant(bits, sh)];
+  pdl_wait();
   const int M = (int)sh.M, K = sh.K, N = sh.N;
   const bool unit_in = it.in_rec < 0;
   const float mu = unit_in ? 1.f : __uint_as_float(recs[it.in_rec].maxbits);
@@ -425,8 +429,8 @@ cudaError_t launch_cfg(const SimtParams &p, const StepItem *items, int n_items, 
   // row tiles per block: as many as leave the chip about eight blocks per SM
   const int64_t per = mt * nt * (int64_t)n_items / (8 * 152);
   if (per > 1) mt = (mt + per - 1) / per;
-  kern<<<dim3((unsigned)mt, nt, n_items), THREADS, smem, s>>>(p, items, ops, recs);
-  return cudaGetLastError();
+  return launch_dependent(kern, dim3((unsigned)mt, nt, n_items), dim3(THREADS), smem, s, p, items, ops,
+                          recs);
 }
 
 // The tile of a launch: 128 rows x 64 columns where that gives two waves of two
@@ -505,15 +509,14 @@ cudaError_t launch_contract_simt(const StepShape &sh, const StepItem *d_items, i
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidValue;
     dim3 grid((unsigned)blocks, n_items);
     switch (sh.fmt) {
-      case FMT_F32: k_contract_rows<FMT_F32><<<grid, 256, 0, s>>>(sh, d_items, d_ops, d_recs); break;
-      case FMT_TF32: k_contract_rows<FMT_TF32><<<grid, 256, 0, s>>>(sh, d_items, d_ops, d_recs); break;
-      case FMT_BF16: k_contract_rows<FMT_BF16><<<grid, 256, 0, s>>>(sh, d_items, d_ops, d_recs); break;
-      case FMT_FP16: k_contract_rows<FMT_FP16><<<grid, 256, 0, s>>>(sh, d_items, d_ops, d_recs); break;
-      case FMT_BF16X2: k_contract_rows<FMT_BF16X2><<<grid, 256, 0, s>>>(sh, d_items, d_ops, d_recs); break;
-      case FMT_FP16X2: k_contract_rows<FMT_FP16X2><<<grid, 256, 0, s>>>(sh, d_items, d_ops, d_recs); break;
-      default: return cudaErrorInvalidValue;
+      case FMT_F32: return launch_dependent(k_contract_rows<FMT_F32>, grid, dim3(256), 0, s, sh, d_items, d_ops, d_recs);
+      case FMT_TF32: return launch_dependent(k_contract_rows<FMT_TF32>, grid, dim3(256), 0, s, sh, d_items, d_ops, d_recs);
+      case FMT_BF16: return launch_dependent(k_contract_rows<FMT_BF16>, grid, dim3(256), 0, s, sh, d_items, d_ops, d_recs);
+      case FMT_FP16: return launch_dependent(k_contract_rows<FMT_FP16>, grid, dim3(256), 0, s, sh, d_items, d_ops, d_recs);
+      case FMT_BF16X2: return launch_dependent(k_contract_rows<FMT_BF16X2>, grid, dim3(256), 0, s, sh, d_items, d_ops, d_recs);
+      case FMT_FP16X2: return launch_dependent(k_contract_rows<FMT_FP16X2>, grid, dim3(256), 0, s, sh, d_items, d_ops, d_recs);
     }
-    return cudaGetLastError();
+    return cudaErrorInvalidValue;
   }
   switch (sh.fmt) {
     case FMT_F32: return launch_tiles<FMT_F32>(sh, d_items, n_items, d_ops, d_recs, aligned32, s);

@@ -464,6 +464,7 @@ __global__ void __launch_bounds__(threads_of(EPI, DR), 1)
   __syncthreads();
   if (CG > 1) cluster_sync();  // both CTAs' barriers exist before any remote signal
   tc_fence_after();
+  pdl_trigger();
   const uint32_t tmem_base = *tmem_slot;
 
   const int cid = blockIdx.x / CG, ncl = gridDim.x / CG;
@@ -478,6 +479,11 @@ __global__ void __launch_bounds__(threads_of(EPI, DR), 1)
   // a row of A holds 2K real entries of ESZ bytes; one stage covers ROWB bytes
   const int kb_count = (2 * p.sh.K * T::ESZ) / ROWB;
   Watch w{abort_flag, p.st, globaltimer() + (uint64_t)p.watchdog_ns, p.sh.q, CG};
+  // the launch before has completed; the waits' budget counts from here
+  auto start_watch = [&]() {
+    pdl_wait();
+    w.deadline = globaltimer() + (uint64_t)p.watchdog_ns;
+  };
   // the even CTA's barriers, as cluster addresses
   const uint32_t full0 = CG == 2 ? cluster_addr(full, 0) : 0u;
   const uint32_t tempty0 = CG == 2 ? cluster_addr(tempty, 0) : 0u;
@@ -490,7 +496,7 @@ __global__ void __launch_bounds__(threads_of(EPI, DR), 1)
     uint32_t it = 0;
     {
       ItemBlock ib{INT32_MIN, 0, 0};
-      bool ok = true;
+      bool ok = true, first = true;
       for (int t = t_first; t < t_end; t += t_step) {
         const int item = (int)p.d_tpi.q(t);
         const int rem = t - item * tiles_per_item;
@@ -508,6 +514,8 @@ __global__ void __launch_bounds__(threads_of(EPI, DR), 1)
           const StepItem &si = p.items[i];
           ib.tau = block_variant(*si.bits, p.sh) + si.b_slot;
           ib.a_lane = si.a_lane;
+          if (first) start_watch();
+          first = false;
         }
         const int tau = __shfl_sync(0xffffffffu, ib.tau, item - ib.base);
         const int a_lane = __shfl_sync(0xffffffffu, ib.a_lane, item - ib.base);
@@ -601,6 +609,7 @@ __global__ void __launch_bounds__(threads_of(EPI, DR), 1)
       const uint32_t idesc = (1u << 4) | ((uint32_t)T::AB << 7) | ((uint32_t)T::AB << 10) |
                              ((uint32_t)(BN >> 3) << 17) | ((uint32_t)((BM * CG) >> 4) << 24);
       uint32_t it = 0, local = 0;
+      start_watch();
       const int KSP = p.ksplit, NB = p.nbuf;
       for (int t = t_first; t < t_end; t += t_step, ++local) {
         const int acc = NB == 2 ? (int)(local & 1) : 0;
@@ -705,6 +714,7 @@ __global__ void __launch_bounds__(threads_of(EPI, DR), 1)
     int cached_item = -1, out_rec = 0, out_exp = 0;
     void *D = nullptr;
     float sc = 1.f, vmax = 0.f;
+    bool first = true;
     // the item's max |entry|, once per item and warp (non-negative floats
     // compare as their bits)
     auto flush_max = [&]() {
@@ -729,8 +739,10 @@ __global__ void __launch_bounds__(threads_of(EPI, DR), 1)
         if (item >= ib_base + 32 || ib_base < 0) {
           ib_base = item;
           const int i = item + lane < p.n_items ? item + lane : item;
-          const StepItem &si = p.items[i];
+          const StepItem si = p.items[i];
           const OpDesc &op = p.ops[si.op_base + block_variant(*si.bits, p.sh)];
+          if (first) start_watch();
+          first = false;
           const bool unit_in = si.in_rec < 0;
           const float mu = unit_in ? 1.f : __uint_as_float(p.recs[si.in_rec].maxbits);
           const int s_in = unit_in ? 0 : p.recs[si.in_rec].exp;
@@ -1377,17 +1389,25 @@ static cudaError_t launch_one(const TcParams &prm, int units, size_t smem, cudaS
   if (max_clusters > 0 && clusters > max_clusters) clusters = max_clusters;
   if (clusters < 1) clusters = 1;
   cudaLaunchConfig_t cfg = {};
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = CG;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  // Dependent launch (pdl_wait), but not for long launches in interleaved or
+  // grouped order: started as SMs come free, the pairs that share k-slabs in L2
+  // land on different dies (512 lanes of the 1024 x 1024 x 256 merge: 1616 us
+  // placed in order, 1849 us so).
+  const bool in_order = !prm.blocked && (int64_t)prm.n_items * (prm.tiles_m / CG) * prm.tiles_n >
+                                            4 * (int64_t)clusters;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.gridDim = dim3(clusters * CG);
   cfg.blockDim = dim3(threads_of(EPI, DR));
   cfg.dynamicSmemBytes = smem;
   cfg.stream = s;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = in_order ? 1 : 2;
   return cudaLaunchKernelEx(&cfg, kern, prm);
 }
 

@@ -11,6 +11,8 @@ namespace peps {
 template <int FMT>
 __global__ void k_finalize(const FinalEntry *__restrict__ entries, int n, int64_t plane,
                            const Rec *__restrict__ recs, double2 *acc) {
+  pdl_trigger();
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const FinalEntry f = entries[i];
@@ -27,15 +29,14 @@ cudaError_t launch_finalize(const FinalEntry *d_entries, int n, int fmt, int64_t
   if (n <= 0) return cudaSuccess;
   const int threads = 128, blocks = (n + threads - 1) / threads;
   switch (fmt) {
-    case FMT_F32: k_finalize<FMT_F32><<<blocks, threads, 0, s>>>(d_entries, n, plane, d_recs, d_acc); break;
-    case FMT_TF32: k_finalize<FMT_TF32><<<blocks, threads, 0, s>>>(d_entries, n, plane, d_recs, d_acc); break;
-    case FMT_BF16: k_finalize<FMT_BF16><<<blocks, threads, 0, s>>>(d_entries, n, plane, d_recs, d_acc); break;
-    case FMT_FP16: k_finalize<FMT_FP16><<<blocks, threads, 0, s>>>(d_entries, n, plane, d_recs, d_acc); break;
-    case FMT_BF16X2: k_finalize<FMT_BF16X2><<<blocks, threads, 0, s>>>(d_entries, n, plane, d_recs, d_acc); break;
-    case FMT_FP16X2: k_finalize<FMT_FP16X2><<<blocks, threads, 0, s>>>(d_entries, n, plane, d_recs, d_acc); break;
-    default: return cudaErrorInvalidValue;
+    case FMT_F32: return launch_dependent(k_finalize<FMT_F32>, dim3(blocks), dim3(threads), 0, s, d_entries, n, plane, d_recs, d_acc);
+    case FMT_TF32: return launch_dependent(k_finalize<FMT_TF32>, dim3(blocks), dim3(threads), 0, s, d_entries, n, plane, d_recs, d_acc);
+    case FMT_BF16: return launch_dependent(k_finalize<FMT_BF16>, dim3(blocks), dim3(threads), 0, s, d_entries, n, plane, d_recs, d_acc);
+    case FMT_FP16: return launch_dependent(k_finalize<FMT_FP16>, dim3(blocks), dim3(threads), 0, s, d_entries, n, plane, d_recs, d_acc);
+    case FMT_BF16X2: return launch_dependent(k_finalize<FMT_BF16X2>, dim3(blocks), dim3(threads), 0, s, d_entries, n, plane, d_recs, d_acc);
+    case FMT_FP16X2: return launch_dependent(k_finalize<FMT_FP16X2>, dim3(blocks), dim3(threads), 0, s, d_entries, n, plane, d_recs, d_acc);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 // Square partition, last contraction: sum_i Y[i] F[i] for each entry.  Pass
@@ -53,7 +54,9 @@ cudaError_t launch_finalize(const FinalEntry *d_entries, int n, int fmt, int64_t
 template <int FMT>
 __global__ void __launch_bounds__(256) k_dot(const DotEntry *__restrict__ entries, int64_t plane,
                                              double2 *partials) {
+  pdl_trigger();
   const DotEntry d = entries[blockIdx.y];
+  pdl_wait();
   float re0 = 0.f, im0 = 0.f, re1 = 0.f, im1 = 0.f;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -90,8 +93,10 @@ __global__ void __launch_bounds__(128) k_dot_final(const DotEntry *__restrict__ 
                                                    const Rec *__restrict__ recs,
                                                    const double2 *__restrict__ partials,
                                                    double2 *acc) {
+  pdl_trigger();
   const int e = blockIdx.x;
   const DotEntry d = entries[e];
+  pdl_wait();
   const int ns = d.nslots;
   double re = 0.0, im = 0.0;
   for (int b = threadIdx.x; b < ns; b += blockDim.x) {
@@ -122,26 +127,23 @@ cudaError_t launch_dot(const DotEntry *d_entries, int n, int fmt, int64_t plane,
                        const Rec *d_recs, double2 *d_partials, double2 *d_acc, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const dim3 grid(kDotBlocks, n);
+  cudaError_t e = cudaErrorInvalidValue;
   switch (fmt) {
-    case FMT_F32: k_dot<FMT_F32><<<grid, 256, 0, s>>>(d_entries, plane, d_partials); break;
-    case FMT_TF32: k_dot<FMT_TF32><<<grid, 256, 0, s>>>(d_entries, plane, d_partials); break;
-    case FMT_BF16: k_dot<FMT_BF16><<<grid, 256, 0, s>>>(d_entries, plane, d_partials); break;
-    case FMT_FP16: k_dot<FMT_FP16><<<grid, 256, 0, s>>>(d_entries, plane, d_partials); break;
-    case FMT_BF16X2: k_dot<FMT_BF16X2><<<grid, 256, 0, s>>>(d_entries, plane, d_partials); break;
-    case FMT_FP16X2: k_dot<FMT_FP16X2><<<grid, 256, 0, s>>>(d_entries, plane, d_partials); break;
-    default: return cudaErrorInvalidValue;
+    case FMT_F32: e = launch_dependent(k_dot<FMT_F32>, grid, dim3(256), 0, s, d_entries, plane, d_partials); break;
+    case FMT_TF32: e = launch_dependent(k_dot<FMT_TF32>, grid, dim3(256), 0, s, d_entries, plane, d_partials); break;
+    case FMT_BF16: e = launch_dependent(k_dot<FMT_BF16>, grid, dim3(256), 0, s, d_entries, plane, d_partials); break;
+    case FMT_FP16: e = launch_dependent(k_dot<FMT_FP16>, grid, dim3(256), 0, s, d_entries, plane, d_partials); break;
+    case FMT_BF16X2: e = launch_dependent(k_dot<FMT_BF16X2>, grid, dim3(256), 0, s, d_entries, plane, d_partials); break;
+    case FMT_FP16X2: e = launch_dependent(k_dot<FMT_FP16X2>, grid, dim3(256), 0, s, d_entries, plane, d_partials); break;
   }
-  cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
-  k_dot_final<<<n, 128, 0, s>>>(d_entries, d_recs, d_partials, d_acc);
-  return cudaGetLastError();
+  return launch_dot_final(d_entries, n, d_recs, d_partials, d_acc, s);
 }
 
 cudaError_t launch_dot_final(const DotEntry *d_entries, int n, const Rec *d_recs,
                              const double2 *d_partials, double2 *d_acc, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  k_dot_final<<<n, 128, 0, s>>>(d_entries, d_recs, d_partials, d_acc);
-  return cudaGetLastError();
+  return launch_dependent(k_dot_final, dim3(n), dim3(128), 0, s, d_entries, d_recs, d_partials, d_acc);
 }
 
 __global__ void k_store_out(const double2 *__restrict__ acc, peps_c128 *out, int64_t n) {

@@ -10,6 +10,33 @@
 
 namespace peps {
 
+// Programmatic dependent launch.  A contraction chain is hundreds of short
+// kernels, each waiting for the one before; a kernel launched with
+// launch_dependent starts while the kernel before it on the stream still runs
+// (once that one's blocks have all called pdl_trigger), sets itself up, and
+// reads or writes what kernels produce only after pdl_wait, which returns when
+// the kernel before has completed.  Every kernel launched this way calls both,
+// so completion stays in stream order.  Before pdl_wait only the plan's
+// tables (items) and the bitstrings may be read: they are copied in before the
+// call's first kernel.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+template <class... P, class... A>
+inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, size_t smem,
+                                    cudaStream_t s, A... args) {
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, P(args)...);
+}
+
 // x / d and x % d for a divisor fixed per launch (1 <= d <= 2^31, 0 <= x <
 // 2^31), branch-free: q = (mulhi(m, x) + x) >> l with l = ceil(log2 d) and
 // m = floor(2^32 (2^l - d) / d) + 1 (Granlund and Montgomery, "Division by
