@@ -2368,7 +2368,7 @@ static int enqueue_sequence_stats_only(Plan &P, peps_stats &S) {
         S.contract_tc_bytes += k * l.bytes;
       }
     } else if (l.kind == 2) {
-      S.launches_operand += k * (l.tc ? 3 : 2);
+      S.launches_operand += k * 2;
     } else if (l.kind == 3) {
       S.launches_finalize += (l.fused_merge >= 0 ? 1 : 2) * k;
     } else {
@@ -2512,13 +2512,12 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
         if (l.tc) {
           CUDA_TRY(launch_tensor_operand_tc(tops + l.aux_off, l.n_aux, l.shape.K, l.shape.N, P.fmt,
                                             P.plane, ops, recs, s));
-          S.launches_operand += 3;
         } else {
           CUDA_TRY(launch_tensor_operand(tops + l.aux_off, l.n_aux, l.kn, P.fmt, P.plane, ops, recs,
                                          s));
           CUDA_TRY(launch_operand_bounds(l.n_aux, ops + l.op, s, l.shape.N));
-          S.launches_operand += 2;
         }
+        S.launches_operand += 2;
       } else if (l.kind == 3 && l.fused_merge >= 0) {
         CUDA_TRY(launch_dot_final(dots + l.aux_off, l.n_aux, recs, partials, acc, s));
         S.launches_finalize += 1;

@@ -1542,12 +1542,15 @@ __global__ void __launch_bounds__(256) k_build_bt(OpDesc *ops) {
 
 // A merge operand straight from a stored tensor G whose k index is contiguous:
 // Ec[k][n] = G[k + nh ns_hi + nl ns] 2^-target (n = nh Nlo + nl) is never
-// written out.  k_tensor_bound takes the column bound beta_c = max_n
-// sum_k |Ec[k][n]|_1 (one block per column, the threads along k), k_tensor_bt
-// the complex-as-real planes Bt[(n, b)][(k, a)] (reads and writes both run
-// along k).  Same values as Ec -> k_beta_ops -> k_build_bt.
+// written out.  One pass over G gives the column bound beta_c = max_n sum_k
+// |Ec[k][n]|_1 and the complex-as-real planes Bt[(n, b)][(k, a)]; reads and
+// writes both run along k.  Bound by memory: 8 bytes read and 16 written per
+// entry (FP16X3).  16 operands of 4096 x 4096: bound and planes in two passes
+// 2380 us, in this one 1086 us (5.9 TB/s).  Same values as Ec -> k_beta_ops -> k_build_bt.
 __global__ void k_tensor_init(const TensorOpEntry *__restrict__ e, int n, OpDesc *ops,
                               const Rec *recs) {
+  pdl_trigger();
+  pdl_wait();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const TensorOpEntry g = e[i];
@@ -1557,115 +1560,135 @@ __global__ void k_tensor_init(const TensorOpEntry *__restrict__ e, int n, OpDesc
   op.e_c = recs[g.rec].exp - g.target;
 }
 
+// Entry k of column n (ek = its value 2^-target 2^b_t) into both rows of the planes.
 template <int FMT>
-__global__ void __launch_bounds__(256) k_tensor_bound(const TensorOpEntry *__restrict__ e,
-                                                      int64_t plane, OpDesc *ops) {
+__device__ __forceinline__ void put_bt(void *hi, void *lo, int64_t n, int64_t K, int64_t k,
+                                       float re, float im) {
+  // row 2n holds (re, -im) at columns 2k, 2k+1; row 2n+1 holds (im, re)
+  const float2 r0 = make_float2(re, -im), r1 = make_float2(im, re);
+  const int64_t w0 = 2 * n * K + k, w1 = w0 + K;   // in column pairs
+  if (FMT == FMT_TF32) {
+    ((float2 *)hi)[w0] = make_float2(round_tf32(r0.x), round_tf32(r0.y));
+    ((float2 *)hi)[w1] = make_float2(round_tf32(r1.x), round_tf32(r1.y));
+  } else if (FMT == FMT_BF16) {
+    ((uint32_t *)hi)[w0] = pack_bf16(r0.x, r0.y);
+    ((uint32_t *)hi)[w1] = pack_bf16(r1.x, r1.y);
+  } else if (FMT == FMT_FP16) {
+    ((uint32_t *)hi)[w0] = pack_f16(r0.x, r0.y);
+    ((uint32_t *)hi)[w1] = pack_f16(r1.x, r1.y);
+  } else {
+    constexpr bool BF = FMT == FMT_BF16X2;
+    uint32_t h0, l0, h1, l1;
+    split16<BF>(r0, h0, l0);
+    split16<BF>(r1, h1, l1);
+    ((uint32_t *)hi)[w0] = h0;
+    ((uint32_t *)hi)[w1] = h1;
+    ((uint32_t *)lo)[w0] = l0;
+    ((uint32_t *)lo)[w1] = l1;
+  }
+}
+
+// COL = 1: a block per column (threads along k), COL = 0: a warp per column (K
+// too short for a block).  Either way a column's sum is eight partial sums (k
+// mod 256 in [32 w, 32 w + 32), each the tree of 32 lane sums over k ascending)
+// added in order.
+template <int FMT, int COL>
+__global__ void __launch_bounds__(256) k_tensor_bt(const TensorOpEntry *__restrict__ e,
+                                                   int64_t plane, OpDesc *ops) {
+  pdl_trigger();
   const TensorOpEntry g = e[blockIdx.y];   // one entry per grid row
-  const float sc = pow2f(-g.target);
+  pdl_wait();
+  OpDesc &op = ops[g.op];
+  const int64_t K = g.K, N = g.N;
+  void *const hi = const_cast<void *>(op.Bt[0]), *const lo = const_cast<void *>(op.Bt[1]);
+  const float sc = pow2f(-g.target), sb = ldexpf(1.f, op.b_t);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   __shared__ float red[8];
   float best = 0.f;
-  for (int64_t n = blockIdx.x; n < g.N; n += gridDim.x) {
-    const int64_t nh = n / g.Nlo, nl = n - nh * g.Nlo;
-    const int64_t base = nh * g.ns_hi + nl * g.ns;
+  // the lane sum over k = k0, k0 + 256, ..., four loads in flight
+  auto lane_sum = [&](int64_t n, int64_t base, int64_t k0) {
     float s = 0.f;
-    for (int64_t k = threadIdx.x; k < g.K; k += blockDim.x) {
-      const float2 v = load_g<FMT>(g.G, base + k * g.ks, plane);
-      s += fabsf(v.x * sc) + fabsf(v.y * sc);
+    for (int64_t k = k0; k < K; k += 1024) {
+      float2 v[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u)
+        if (k + 256 * u < K) v[u] = load_g<FMT>(g.G, base + (k + 256 * u) * g.ks, plane);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        if (k + 256 * u >= K) break;
+        const float re = v[u].x * sc, im = v[u].y * sc;
+        s += fabsf(re) + fabsf(im);
+        put_bt<FMT>(hi, lo, n, K, k + 256 * u, re * sb, im * sb);
+      }
     }
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
+    return s;
+  };
+  auto column = [&](int64_t n) {
+    const int64_t nh = n / g.Nlo, nl = n - nh * g.Nlo;
+    return nh * g.ns_hi + nl * g.ns;
+  };
+  if (COL) {
+    for (int64_t n = blockIdx.x; n < N; n += gridDim.x) {
+      const float s = lane_sum(n, column(n), threadIdx.x);
+      if (lane == 0) red[warp] = s;
+      __syncthreads();
+      if (threadIdx.x == 0) {
+        float t = 0.f;
+        for (int w = 0; w < 8; ++w) t += red[w];
+        best = fmaxf(best, t);
+      }
+      __syncthreads();
+    }
+  } else {
+    for (int64_t n = (int64_t)blockIdx.x * 8 + warp; n < N; n += (int64_t)gridDim.x * 8) {
+      const int64_t base = column(n);
       float t = 0.f;
-      for (int w = 0; w < 8; ++w) t += red[w];
+      for (int w = 0; w < 8 && 32 * w < K; ++w) t += lane_sum(n, base, 32 * w + lane);
       best = fmaxf(best, t);
     }
+    if (lane == 0) red[warp] = best;
     __syncthreads();
+    if (threadIdx.x == 0)
+      for (int w = 0; w < 8; ++w) best = fmaxf(best, red[w]);
   }
-  if (threadIdx.x == 0)
-    atomicMax(&ops[g.op].beta_c_bits, __float_as_uint(best * (1.0f + 1.0f / 256.0f)));
+  if (threadIdx.x == 0) {
+    // beta_t = beta_c 2^b_t with its margin: increasing in beta_c, so the
+    // blocks' largest is that of the largest beta_c
+    const float bc = best * (1.0f + 1.0f / 256.0f);
+    atomicMax(&op.beta_c_bits, __float_as_uint(bc));
+    atomicMax(&op.beta_t_bits, __float_as_uint(bc * sb * (1.0f + 1.0f / 128.0f)));
+  }
 }
 
 template <int FMT>
-__global__ void k_tensor_bt(const TensorOpEntry *__restrict__ e, int64_t plane, OpDesc *ops) {
-  const TensorOpEntry g = e[blockIdx.y];   // one entry per grid row
-  OpDesc &op = ops[g.op];
-  const int64_t K = g.K, N = g.N;
-  const float sc = pow2f(-g.target), sb = ldexpf(1.f, op.b_t);
-  const bool narrow = K * N < ((int64_t)1 << 31) && g.Nlo < ((int64_t)1 << 31);
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < K * N;
-       i += (int64_t)gridDim.x * blockDim.x) {
-    int64_t n, k, nh, nl;
-    if (narrow) {   // 32-bit index arithmetic
-      const uint32_t i32 = (uint32_t)i, n32 = i32 / (uint32_t)K, lo = (uint32_t)g.Nlo;
-      n = n32;
-      k = i32 - n32 * (uint32_t)K;
-      nh = n32 / lo;
-      nl = n32 - (uint32_t)nh * lo;
-    } else {
-      n = i / K;
-      k = i - n * K;
-      nh = n / g.Nlo;
-      nl = n - nh * g.Nlo;
-    }
-    const float2 v = load_g<FMT>(g.G, k * g.ks + nh * g.ns_hi + nl * g.ns, plane);
-    const float re = (v.x * sc) * sb, im = (v.y * sc) * sb;
-    // row 2n holds (re, -im) at columns 2k, 2k+1; row 2n+1 holds (im, re)
-    const float2 r0 = make_float2(re, -im), r1 = make_float2(im, re);
-    const int64_t w0 = 2 * n * K + k, w1 = (2 * n + 1) * K + k;   // in column pairs
-    if (FMT == FMT_TF32) {
-      ((float2 *)op.Bt[0])[w0] = make_float2(round_tf32(r0.x), round_tf32(r0.y));
-      ((float2 *)op.Bt[0])[w1] = make_float2(round_tf32(r1.x), round_tf32(r1.y));
-    } else if (FMT == FMT_BF16) {
-      ((uint32_t *)op.Bt[0])[w0] = pack_bf16(r0.x, r0.y);
-      ((uint32_t *)op.Bt[0])[w1] = pack_bf16(r1.x, r1.y);
-    } else if (FMT == FMT_FP16) {
-      ((uint32_t *)op.Bt[0])[w0] = pack_f16(r0.x, r0.y);
-      ((uint32_t *)op.Bt[0])[w1] = pack_f16(r1.x, r1.y);
-    } else {
-      constexpr bool BF = FMT == FMT_BF16X2;
-      uint32_t h0, l0, h1, l1;
-      split16<BF>(r0, h0, l0);
-      split16<BF>(r1, h1, l1);
-      ((uint32_t *)op.Bt[0])[w0] = h0;
-      ((uint32_t *)op.Bt[0])[w1] = h1;
-      ((uint32_t *)op.Bt[1])[w0] = l0;
-      ((uint32_t *)op.Bt[1])[w1] = l1;
-    }
-  }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    const float bc = __uint_as_float(op.beta_c_bits);
-    op.beta_t_bits = __float_as_uint(bc * sb * (1.0f + 1.0f / 128.0f));
-  }
+static cudaError_t tensor_bt(const TensorOpEntry *d_entry, int n_entries, int K, int N,
+                             int64_t plane, OpDesc *d_ops, cudaStream_t s) {
+  // some 16 blocks per SM in all, each with several columns
+  const bool col = K >= 1024;
+  const int units = col ? N : (N + 7) / 8;
+  int gx = (16 * 152 + n_entries - 1) / n_entries;
+  if (gx > units) gx = units;
+  const dim3 grid((unsigned)gx, (unsigned)n_entries);
+  return col ? launch_dependent(k_tensor_bt<FMT, 1>, grid, dim3(256), 0, s, d_entry, plane, d_ops)
+             : launch_dependent(k_tensor_bt<FMT, 0>, grid, dim3(256), 0, s, d_entry, plane, d_ops);
 }
 
 cudaError_t launch_tensor_operand_tc(const TensorOpEntry *d_entry, int n_entries, int K, int N,
                                      int fmt, int64_t plane, OpDesc *d_ops, const Rec *d_recs,
                                      cudaStream_t s) {
   if (n_entries <= 0) return cudaSuccess;
-  const int64_t kn = (int64_t)K * N;
-  int64_t gb = N < 16384 ? N : 16384;
-  if (gb < 1) gb = 1;
-  int64_t gt = (kn + 255) / 256;
-  if (gt > 16384) gt = 16384;
-  if (gt < 1) gt = 1;
-  k_tensor_init<<<(n_entries + 127) / 128, 128, 0, s>>>(d_entry, n_entries, d_ops, d_recs);
-  const dim3 grid_b((unsigned)gb, (unsigned)n_entries), grid_t((unsigned)gt, (unsigned)n_entries);
+  const cudaError_t r = launch_dependent(k_tensor_init, dim3((n_entries + 127) / 128), dim3(128), 0, s,
+                                         d_entry, n_entries, d_ops, d_recs);
+  if (r != cudaSuccess) return r;
   switch (fmt) {
-#define PEPS_TOP_CASE(F)                                                              \
-  case F:                                                                            \
-    k_tensor_bound<F><<<grid_b, 256, 0, s>>>(d_entry, plane, d_ops);                 \
-    k_tensor_bt<F><<<grid_t, 256, 0, s>>>(d_entry, plane, d_ops);                    \
-    break;
-    PEPS_TOP_CASE(FMT_TF32)
-    PEPS_TOP_CASE(FMT_BF16)
-    PEPS_TOP_CASE(FMT_FP16)
-    PEPS_TOP_CASE(FMT_BF16X2)
-    PEPS_TOP_CASE(FMT_FP16X2)
-#undef PEPS_TOP_CASE
-    default: return cudaErrorInvalidValue;
+    case FMT_TF32: return tensor_bt<FMT_TF32>(d_entry, n_entries, K, N, plane, d_ops, s);
+    case FMT_BF16: return tensor_bt<FMT_BF16>(d_entry, n_entries, K, N, plane, d_ops, s);
+    case FMT_FP16: return tensor_bt<FMT_FP16>(d_entry, n_entries, K, N, plane, d_ops, s);
+    case FMT_BF16X2: return tensor_bt<FMT_BF16X2>(d_entry, n_entries, K, N, plane, d_ops, s);
+    case FMT_FP16X2: return tensor_bt<FMT_FP16X2>(d_entry, n_entries, K, N, plane, d_ops, s);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_build_tc_operands(int n, int64_t max_kn, OpDesc *d_ops, int fmt,

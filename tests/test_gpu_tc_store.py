@@ -64,15 +64,19 @@ def test_separate_corrections_with_one_accumulator_buffer(cuda_device, prec, tol
     sim.close()
 
 
-def test_bonds_that_are_not_powers_of_two(cuda_device):
+@pytest.mark.parametrize("R,C,layers,n,kw", [
+    (4, 5, 5, 35, dict(max_lanes=35)),
+    (4, 6, 4, 9, dict(scheme="quadrants")),   # a merge operand of 48 x 8
+])
+def test_bonds_that_are_not_powers_of_two(cuda_device, R, C, layers, n, kw):
     from paper_1905_08394_gb300 import Simulator
 
-    circ = make_circuit_general(4, 5, 5, 7)
-    bits = uniform_bitstrings(20, 35, 7)
-    ref = sv.amplitudes(20, circ.gates, bits)
-    sim = Simulator(4, 5, device=cuda_device.index or 0)
+    circ = make_circuit_general(R, C, layers, 7)
+    bits = uniform_bitstrings(R * C, n, 7)
+    ref = sv.amplitudes(R * C, circ.gates, bits)
+    sim = Simulator(R, C, device=cuda_device.index or 0)
     sim.apply_circuit(circ)
-    out = sim.amplitudes(bits, precision="fp16x3", max_lanes=35)
+    out = sim.amplitudes(bits, precision="fp16x3", **kw)
     assert sim.stats()["launches_contract_tc"] > 0
     assert relerr(out, ref) < TOL
     sim.close()
