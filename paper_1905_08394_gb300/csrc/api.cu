@@ -1977,7 +1977,7 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
     }
     off = align_up(off + (quad ? per_lane * P.lanes * sizeof(double2) : 16));
   }
-  P.off_small_steps = off; off = align_up(off + (size_t)std::max(NS, (int64_t)1) * sizeof(StepShape));
+  P.off_small_steps = off; off = align_up(off + (size_t)std::max(NS, (int64_t)1) * sizeof(SmallStep));
   P.off_small_opbase = off; off = align_up(off + (size_t)std::max(NS, (int64_t)1) * sizeof(int32_t));
   P.off_acc = off; off = align_up(off + std::max<int64_t>(n, 1) * sizeof(double2));
   P.off_bits = off; off = align_up(off + std::max<int64_t>(n, 1) * sizeof(uint64_t));
@@ -2211,7 +2211,11 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
   put(P.off_g2, g2e.data(), g2e.size() * sizeof(Gate2Entry));
   put(P.off_evo_refs, evo_refs.data(), evo_refs.size() * sizeof(EvoRef));
   put(P.off_evo_first, evo_first.data(), evo_first.size() * sizeof(int32_t));
-  put(P.off_small_steps, P.steps.data(), P.steps.size() * sizeof(StepShape));
+  if (P.small) {
+    std::vector<SmallStep> ss;
+    for (const auto &sh : P.steps) ss.push_back(small_step(sh));
+    put(P.off_small_steps, ss.data(), ss.size() * sizeof(SmallStep));
+  }
   put(P.off_small_opbase, P.step_opbase.data(), P.step_opbase.size() * sizeof(int32_t));
   put(P.off_opdesc, ops.data(), ops.size() * sizeof(OpDesc));
   put(P.off_opbuild, obe.data(), obe.size() * sizeof(OpBuildEntry));
@@ -2478,7 +2482,7 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
         if (timing) CUDA_TRY(record(c->ev[2 * *n_timed]));
         if (l.small) {
           SmallSweep sw{};
-          sw.steps = (const StepShape *)(base + P.off_small_steps);
+          sw.steps = (const SmallStep *)(base + P.off_small_steps);
           sw.op_base = (const int32_t *)(base + P.off_small_opbase);
           sw.ops = ops;
           sw.bits = P.small_bits;

@@ -53,6 +53,27 @@ inline int operand_scale_exp(int fmt) {
   return (fmt == FMT_FP16 || fmt == FMT_FP16X2) ? 12 : 0;
 }
 
+// x / d and x % d for a divisor fixed per launch (1 <= d <= 2^31, 0 <= x <
+// 2^31), branch-free: q = (mulhi(m, x) + x) >> l with l = ceil(log2 d) and
+// m = floor(2^32 (2^l - d) / d) + 1 (Granlund and Montgomery, "Division by
+// invariant integers using multiplication", 1994).  One form for every
+// divisor: with a branch between a shift and a 64-bit division the division's
+// code lies between the hot instructions, and the tensor-core kernel's tile
+// set-up alone took about 1700 of a 128 x 128 tile's 6200 cycles.
+struct Div {
+  uint32_t d, m;
+  int32_t l;
+  int32_t pad_;
+  __device__ __forceinline__ uint32_t q(uint32_t x) const { return (__umulhi(m, x) + x) >> l; }
+  __device__ __forceinline__ uint32_t r(uint32_t x) const { return x - q(x) * d; }
+};
+inline Div make_div(int64_t d) {
+  Div v{(uint32_t)(d > 0 ? d : 1), 0u, 0, 0};
+  while (((int64_t)1 << v.l) < (int64_t)v.d) ++v.l;
+  v.m = (uint32_t)(((((uint64_t)1 << v.l) - v.d) << 32) / v.d + 1);
+  return v;
+}
+
 // ---------------------------------------------------------------------------
 // Device-side tables
 // ---------------------------------------------------------------------------
@@ -336,8 +357,17 @@ cudaError_t launch_contract_simt(const StepShape &sh, const StepItem *d_items, i
 // the plan's steps and their first operand index, the bitstrings and the
 // FP64 amplitude accumulators; cap_g / cap_e = entries of the largest running
 // tensor / operand (shared memory: two running tensors and one operand).
+struct SmallStep {
+  StepShape sh;
+  int32_t rt, ct;       // thread tile: rows, columns
+  Div d_tn;             // N / ct
+  Div d_Mlo, d_R;       // M / P, the column run (dv', or N where dv' = 1)
+  int32_t R;
+  int32_t stride_q, stride_r;   // of a column run, of a column within it
+  int32_t pad_;
+};
 struct SmallSweep {
-  const StepShape *steps;
+  const SmallStep *steps;
   const int32_t *op_base;
   const OpDesc *ops;
   const uint64_t *bits;
@@ -348,6 +378,7 @@ struct SmallSweep {
   int32_t cap_e;
   int32_t pad_;
 };
+SmallStep small_step(const StepShape &sh);
 constexpr size_t kSmallSweepMaxSmem = 96 * 1024;
 size_t small_sweep_smem(int cap_g, int cap_e);
 cudaError_t launch_sweep_small(const SmallSweep &p, int sm_count, cudaStream_t s);

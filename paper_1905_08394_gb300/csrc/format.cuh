@@ -37,27 +37,6 @@ inline cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, dim3 block, s
   return cudaLaunchKernelEx(&cfg, kern, P(args)...);
 }
 
-// x / d and x % d for a divisor fixed per launch (1 <= d <= 2^31, 0 <= x <
-// 2^31), branch-free: q = (mulhi(m, x) + x) >> l with l = ceil(log2 d) and
-// m = floor(2^32 (2^l - d) / d) + 1 (Granlund and Montgomery, "Division by
-// invariant integers using multiplication", 1994).  One form for every
-// divisor: with a branch between a shift and a 64-bit division the division's
-// code lies between the hot instructions, and the tensor-core kernel's tile
-// set-up alone took about 1700 of a 128 x 128 tile's 6200 cycles.
-struct Div {
-  uint32_t d, m;
-  int32_t l;
-  int32_t pad_;
-  __device__ __forceinline__ uint32_t q(uint32_t x) const { return (__umulhi(m, x) + x) >> l; }
-  __device__ __forceinline__ uint32_t r(uint32_t x) const { return x - q(x) * d; }
-};
-inline Div make_div(int64_t d) {
-  Div v{(uint32_t)(d > 0 ? d : 1), 0u, 0, 0};
-  while (((int64_t)1 << v.l) < (int64_t)v.d) ++v.l;
-  v.m = (uint32_t)(((((uint64_t)1 << v.l) - v.d) << 32) / v.d + 1);
-  return v;
-}
-
 __device__ __forceinline__ float round_tf32(float x) {
   uint32_t r;
   asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
@@ -331,12 +310,33 @@ __device__ __forceinline__ void unpack8(const Raw8 &r, float2 (&f)[8]) {
 // 2^x with x = target - ceil(log2(mu*beta)), which keeps the stored output at
 // most 2^target.  Exact (power of two), deterministic (every CTA computes the
 // same x from the same inputs).
-__device__ __forceinline__ int step_scale_exp(float mu, float beta, int target) {
+//
+// ceil(log2) in integers: the significands' product times 129 (56 bits),
+// rounded to 53 as the double product is; the double form (every thread of a
+// launch evaluates it, and the FP64 pipe takes two lanes a cycle) is left to
+// operands that are zero, subnormal or not finite.
+static __device__ __noinline__ int step_scale_exp_any(float mu, float beta, int target) {
   double p = (double)mu * (double)beta * (1.0 + 1.0 / 128.0);
   if (!(p > 0.0) || !isfinite(p)) return 0;
   int e;
   double f = frexp(p, &e);  // p = f * 2^e, f in [0.5, 1)
   int ce = (f == 0.5) ? e - 1 : e;
+  int x = target - ce;
+  if (x > 120) x = 120;
+  if (x < -120) x = -120;
+  return x;
+}
+__device__ __forceinline__ int step_scale_exp(float mu, float beta, int target) {
+  const uint32_t a = __float_as_uint(mu), b = __float_as_uint(beta);
+  const int ea = (int)(a >> 23), eb = (int)(b >> 23);   // a sign bit makes these >= 256
+  if (ea == 0 || eb == 0 || ea >= 255 || eb >= 255) return step_scale_exp_any(mu, beta, target);
+  const unsigned long long v = (unsigned long long)((a & 0x7fffffu) | 0x800000u) *
+                               ((b & 0x7fffffu) | 0x800000u) * 129ull;
+  const int sh = 64 - __clzll((long long)v) - 53;   // 1 .. 3
+  unsigned long long q = v >> sh;
+  const unsigned long long rem = v & ((1ull << sh) - 1), half = 1ull << (sh - 1);
+  if (rem > half || (rem == half && (q & 1))) ++q;
+  const int ce = 64 - __clzll((long long)q) + sh + ea + eb - 307 - ((q & (q - 1)) == 0 ? 1 : 0);
   int x = target - ce;
   if (x > 120) x = 120;
   if (x < -120) x = -120;
