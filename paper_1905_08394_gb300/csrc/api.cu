@@ -2027,8 +2027,8 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
             (int64_t)(P.bt_off[pl][ob + t] - P.bt_off[pl][ob]) != (int64_t)t * vst)
           return fail(PEPS_EINVAL, "internal: operand variants not equally spaced at site %d", q);
     int rc = tc_prepare(l.shape, fmt, base + P.lane_off + l.a_base_rel, l.a_lanes,
-                        (int64_t)(BPL * P.gbuf_bytes), P.plane * 2, bb, nv, vst, o.tc_kchunk,
-                        o.tc_cluster, o.tc_epi, &l.tc_handle);
+                        (int64_t)(BPL * P.gbuf_bytes), P.plane * 2, bb, nv, vst, l.n_items,
+                        o.tc_kchunk, o.tc_cluster, o.tc_epi, &l.tc_handle);
     if (rc != 0)
       return fail(PEPS_ECUDA, "tensor-map encoding failed (%d) for the step at site %d", rc, q);
   }

@@ -396,10 +396,10 @@ bool tc_tuning_valid(int kchunk, int cluster, int epi);
 // Encode the launch's tensor maps (A over the lanes' input buffers, Bt for
 // tau = 0/1 and each plane); returns 0 and an opaque handle, or < 0.
 // The B operands: plane pl of variant t at b_base[pl] + t * b_var_stride
-// bytes (n_var variants, equally spaced).
+// bytes (n_var variants, equally spaced); n_items: items of the launch.
 int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
                int64_t a_lane_stride, int64_t plane_stride_bytes, const void *const b_base[2],
-               int n_var, int64_t b_var_stride, int kchunk, int cluster, int epi,
+               int n_var, int64_t b_var_stride, int n_items, int kchunk, int cluster, int epi,
                void **out_handle);
 void tc_release(void *handle);
 // One-time set-up of the kernel a handle launches (attributes, occupancy);
