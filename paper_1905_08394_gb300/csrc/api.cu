@@ -168,6 +168,10 @@ struct Plan {
   // first slice builds every operand, a later one only those whose
   // restriction differs from the slice before it)
   std::vector<int64_t> obe_first, obe_count, obe2_first, obe2_count;
+  // the operands those builds write (bounds and planes follow for these only)
+  std::vector<int64_t> ol_first, ol_count;
+  size_t off_oplist = 0;
+  int max_n_site = 1;           // widest site operand (N)
   int max_kn = 0;
   std::vector<int64_t> slice_list;
   double flops_per_slice = 0, bytes_per_slice = 0;
@@ -1581,6 +1585,7 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
       P.max_kn2 = std::max<int>(P.max_kn2, sh.K * sh.N);
       n2 += step_variants(sh);
     }  // nq == 0: a merge operand, built from a stored tensor during the call
+    if (sh.nq > 0) P.max_n_site = std::max(P.max_n_site, sh.N);
     // a tensor-core merge builds its planes straight from the stored tensor
     const bool merge_tc = sh.nq == 0 && want_tc && tc_supports(sh, fmt);
     for (int t = 0; t < op_slots(P, s); ++t) {
@@ -1608,6 +1613,8 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
   off = align_up(off + (size_t)std::max<int64_t>(n1, 1) * P.slice_list.size() * sizeof(OpBuildEntry));
   P.off_opbuild2 = off;
   off = align_up(off + (size_t)std::max<int64_t>(n2, 1) * P.slice_list.size() * sizeof(OpBuild2Entry));
+  P.off_oplist = off;
+  off = align_up(off + (size_t)std::max<int64_t>(n1 + n2, 1) * P.slice_list.size() * sizeof(int32_t));
 
   // records: chains = groups + bitstrings
   P.n_recs = (int)((P.n_groups + n) * P.n_steps);
@@ -2164,6 +2171,7 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
     }
   }
   // keep, for each slice after the first, only the entries that change
+  std::vector<int32_t> oplist;
   {
     const size_t n1 = (size_t)P.n_opbuild_per_slice, n2 = (size_t)P.n_obe2_per_slice;
     const size_t ns = P.slice_list.size();
@@ -2173,6 +2181,8 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
     P.obe_count.assign(ns, 0);
     P.obe2_first.assign(ns, 0);
     P.obe2_count.assign(ns, 0);
+    P.ol_first.assign(ns, 0);
+    P.ol_count.assign(ns, 0);
     for (size_t si = 0; si < ns; ++si) {
       P.obe_first[si] = (int64_t)c1.size();
       for (size_t j = 0; j < n1; ++j) {
@@ -2188,6 +2198,10 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
           c2.push_back(e);
       }
       P.obe2_count[si] = (int64_t)c2.size() - P.obe2_first[si];
+      P.ol_first[si] = (int64_t)oplist.size();
+      for (int64_t j = P.obe_first[si]; j < (int64_t)c1.size(); ++j) oplist.push_back(c1[j].op);
+      for (int64_t j = P.obe2_first[si]; j < (int64_t)c2.size(); ++j) oplist.push_back(c2[j].op);
+      P.ol_count[si] = (int64_t)oplist.size() - P.ol_first[si];
     }
     obe.swap(c1);
     obe2.swap(c2);
@@ -2220,6 +2234,7 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
   put(P.off_opdesc, ops.data(), ops.size() * sizeof(OpDesc));
   put(P.off_opbuild, obe.data(), obe.size() * sizeof(OpBuildEntry));
   put(P.off_opbuild2, obe2.data(), obe2.size() * sizeof(OpBuild2Entry));
+  put(P.off_oplist, oplist.data(), oplist.size() * sizeof(int32_t));
   put(P.off_items, items.data(), items.size() * sizeof(StepItem));
   put(P.off_fin, fins.data(), fins.size() * sizeof(FinalEntry));
   put(P.off_tops, tops.data(), tops.size() * sizeof(TensorOpEntry));
@@ -2356,9 +2371,9 @@ static int enqueue_sequence_stats_only(Plan &P, peps_stats &S) {
   bool any_tc = false;
   for (auto &l : P.launches) any_tc |= (l.kind == 0 && l.tc);
   const int64_t ns = (int64_t)P.slice_list.size();
-  S.launches_operand = ns * (1 + (any_tc ? 1 : 0));
   for (int64_t si = 0; si < ns; ++si)
-    S.launches_operand += (P.obe_count[si] > 0 ? 1 : 0) + (P.obe2_count[si] > 0 ? 1 : 0);
+    S.launches_operand += (P.obe_count[si] > 0 ? 1 : 0) + (P.obe2_count[si] > 0 ? 1 : 0) +
+                          (P.ol_count[si] > 0 ? 1 + (any_tc ? 1 : 0) : 0);
   const int64_t nl = lower_runs(P);
   for (auto &l : P.launches) {
     const int64_t k = l.lower ? nl : ns;
@@ -2470,11 +2485,15 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
       CUDA_TRY(launch_build_operands2(e2, (int)P.obe2_count[si], P.max_kn2, ops, s));
       S.launches_operand++;
     }
-    CUDA_TRY(launch_operand_bounds(P.n_site_ops, ops, s));
-    S.launches_operand++;
-    if (any_tc) {
-      CUDA_TRY(launch_build_tc_operands(P.n_site_ops, std::max(P.max_kn, P.max_kn2), ops, P.fmt, s));
+    const int32_t *ol = (const int32_t *)(base + P.off_oplist) + P.ol_first[si];
+    const int n_ol = (int)P.ol_count[si];
+    if (n_ol > 0) {
+      CUDA_TRY(launch_operand_bounds(n_ol, ol, ops, s, P.max_n_site));
       S.launches_operand++;
+      if (any_tc) {
+        CUDA_TRY(launch_build_tc_operands(n_ol, ol, std::max(P.max_kn, P.max_kn2), ops, P.fmt, s));
+        S.launches_operand++;
+      }
     }
     for (auto &l : P.launches) {
       if (skip_lower && l.lower) continue;
@@ -2519,7 +2538,7 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
         } else {
           CUDA_TRY(launch_tensor_operand(tops + l.aux_off, l.n_aux, l.kn, P.fmt, P.plane, ops, recs,
                                          s));
-          CUDA_TRY(launch_operand_bounds(l.n_aux, ops + l.op, s, l.shape.N));
+          CUDA_TRY(launch_operand_bounds(l.n_aux, nullptr, ops + l.op, s, l.shape.N));
         }
         S.launches_operand += 2;
       } else if (l.kind == 3 && l.fused_merge >= 0) {

@@ -327,9 +327,10 @@ cudaError_t launch_cz(const CzEntry *d_entries, int n, int64_t max_out, cudaStre
 cudaError_t launch_gate2(const Gate2Entry *d_entries, int n, int64_t max_out, cudaStream_t s);
 cudaError_t launch_build_operands(const OpBuildEntry *d_entries, int n, int max_kn,
                                   OpDesc *d_ops, cudaStream_t s);
-// `n_cols`: the widest operand's N (sizes the grid of a single op)
-cudaError_t launch_operand_bounds(int n_ops, OpDesc *d_ops, cudaStream_t s,
-                                  int64_t n_cols = 4096);
+// Bounds of the listed ops (d_list null: ops 0 .. n_ops - 1); `n_cols`: the
+// widest operand's N.
+cudaError_t launch_operand_bounds(int n_ops, const int32_t *d_list, OpDesc *d_ops, cudaStream_t s,
+                                  int64_t n_cols);
 cudaError_t launch_tensor_operand(const TensorOpEntry *d_entries, int n_entries, int64_t kn,
                                   int fmt, int64_t plane, OpDesc *d_ops, const Rec *d_recs,
                                   cudaStream_t s);
@@ -347,9 +348,9 @@ cudaError_t launch_build_operands2(const OpBuild2Entry *d_entries, int n, int ma
 cudaError_t launch_tensor_operand_tc(const TensorOpEntry *d_entries, int n_entries, int K, int N,
                                      int fmt, int64_t plane, OpDesc *d_ops, const Rec *d_recs,
                                      cudaStream_t s);
-// Tensor-core planes (and their bound) of ops [0, n_ops) from their Ec.
-cudaError_t launch_build_tc_operands(int n_ops, int64_t max_kn, OpDesc *d_ops, int fmt,
-                                     cudaStream_t s);
+// Tensor-core planes (and their bound) of the listed ops from their Ec.
+cudaError_t launch_build_tc_operands(int n_ops, const int32_t *d_list, int64_t max_kn,
+                                     OpDesc *d_ops, int fmt, cudaStream_t s);
 cudaError_t launch_contract_simt(const StepShape &sh, const StepItem *d_items, int n_items,
                                  const OpDesc *d_ops, Rec *d_recs, const DeviceStatus *st,
                                  cudaStream_t s, bool aligned32);

@@ -1496,11 +1496,13 @@ cudaError_t launch_contract_tc(void *handle, const StepItem *d_items, int n_item
 // into the form's planes, K-major [Nr][Kr].  Also the bound beta_t.
 // ---------------------------------------------------------------------------
 template <int FMT>
-__global__ void __launch_bounds__(256) k_build_bt(OpDesc *ops) {
-  OpDesc &op = ops[blockIdx.y];
+__global__ void __launch_bounds__(256) k_build_bt(const int32_t *__restrict__ list, OpDesc *ops) {
+  OpDesc &op = ops[list[blockIdx.y]];
   if (op.Bt[0] == nullptr) return;
   const int K = op.K, N = op.N;
   const float sc = ldexpf(1.f, op.b_t);
+  const float2 *const Ec = op.Ec;
+  void *const hi = const_cast<void *>(op.Bt[0]), *const lo = const_cast<void *>(op.Bt[1]);
   // 32 x 32 complex tiles of Ec through shared memory: read along n, written
   // along k, two real columns (a = 0, 1 of one k) per store
   __shared__ float2 tile[32][33];
@@ -1510,10 +1512,33 @@ __global__ void __launch_bounds__(256) k_build_bt(OpDesc *ops) {
     const int k0 = (t / tn) * 32, n0 = (t % tn) * 32;
     for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
       const int kk = e >> 5, nn = e & 31;
-      tile[kk][nn] = (k0 + kk < K && n0 + nn < N) ? op.Ec[(int64_t)(k0 + kk) * N + n0 + nn]
+      tile[kk][nn] = (k0 + kk < K && n0 + nn < N) ? Ec[(int64_t)(k0 + kk) * N + n0 + nn]
                                                     : make_float2(0.f, 0.f);
     }
     __syncthreads();
+    if (FMT != FMT_TF32 && K % 4 == 0) {
+      // four neighbouring k per thread: 16-byte stores, four rows per warp
+      const int k4 = (threadIdx.x & 7) * 4;
+      for (int r = threadIdx.x >> 3; r < 64; r += blockDim.x >> 3) {
+        const int nn = r >> 1, b = r & 1, n = n0 + nn;
+        if (k0 + k4 >= K || n >= N) continue;
+        uint32_t h[4], l[4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          const float2 e = tile[k4 + j][nn];
+          const float v0 = (b == 0 ? e.x : e.y) * sc, v1 = (b == 0 ? -e.y : e.x) * sc;
+          if (FMT == FMT_BF16) h[j] = pack_bf16(v0, v1);
+          else if (FMT == FMT_FP16) h[j] = pack_f16(v0, v1);
+          else split16<FMT == FMT_BF16X2>(make_float2(v0, v1), h[j], l[j]);
+        }
+        const int64_t w = (((int64_t)(2 * n + b) * Kr) >> 1) + k0 + k4;   // in column pairs
+        *(uint4 *)((uint32_t *)hi + w) = make_uint4(h[0], h[1], h[2], h[3]);
+        if (FMT == FMT_BF16X2 || FMT == FMT_FP16X2)
+          *(uint4 *)((uint32_t *)lo + w) = make_uint4(l[0], l[1], l[2], l[3]);
+      }
+      __syncthreads();
+      continue;
+    }
     const int kk = threadIdx.x & 31, k = k0 + kk;
     for (int r = threadIdx.x >> 5; r < 64; r += blockDim.x >> 5) {
       const int nn = r >> 1, b = r & 1, n = n0 + nn;
@@ -1523,17 +1548,17 @@ __global__ void __launch_bounds__(256) k_build_bt(OpDesc *ops) {
       const float v0 = (b == 0 ? e.x : e.y) * sc, v1 = (b == 0 ? -e.y : e.x) * sc;
       const int64_t w = ((int64_t)(2 * n + b) * Kr + 2 * (int64_t)k) >> 1;   // in column pairs
       if (FMT == FMT_TF32) {
-        ((float2 *)op.Bt[0])[w] = make_float2(round_tf32(v0), round_tf32(v1));
+        ((float2 *)hi)[w] = make_float2(round_tf32(v0), round_tf32(v1));
       } else if (FMT == FMT_BF16) {
-        ((uint32_t *)op.Bt[0])[w] = pack_bf16(v0, v1);
+        ((uint32_t *)hi)[w] = pack_bf16(v0, v1);
       } else if (FMT == FMT_FP16) {
-        ((uint32_t *)op.Bt[0])[w] = pack_f16(v0, v1);
+        ((uint32_t *)hi)[w] = pack_f16(v0, v1);
       } else {
         constexpr bool BF = FMT == FMT_BF16X2;
         uint32_t h, l;
         split16<BF>(make_float2(v0, v1), h, l);
-        ((uint32_t *)op.Bt[0])[w] = h;
-        ((uint32_t *)op.Bt[1])[w] = l;
+        ((uint32_t *)hi)[w] = h;
+        ((uint32_t *)lo)[w] = l;
       }
     }
     __syncthreads();
@@ -1697,20 +1722,21 @@ cudaError_t launch_tensor_operand_tc(const TensorOpEntry *d_entry, int n_entries
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_build_tc_operands(int n, int64_t max_kn, OpDesc *d_ops, int fmt,
-                                     cudaStream_t s) {
+cudaError_t launch_build_tc_operands(int n, const int32_t *d_list, int64_t max_kn, OpDesc *d_ops,
+                                     int fmt, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  // 32 x 32 tiles of the largest operand (ops with fewer tiles leave early)
+  // 32 x 32 tiles of the largest operand, up to 128 blocks each (blocks of
+  // smaller operands leave at once, which thousands of them make felt)
   int64_t blocks = (max_kn + 1023) / 1024 + 2;
-  if (blocks > 1024) blocks = 1024;
+  if (blocks > 128) blocks = 128;
   if (blocks < 1) blocks = 1;
   dim3 grid(blocks, n);
   switch (fmt) {
-    case FMT_TF32: k_build_bt<FMT_TF32><<<grid, 256, 0, s>>>(d_ops); break;
-    case FMT_BF16: k_build_bt<FMT_BF16><<<grid, 256, 0, s>>>(d_ops); break;
-    case FMT_FP16: k_build_bt<FMT_FP16><<<grid, 256, 0, s>>>(d_ops); break;
-    case FMT_BF16X2: k_build_bt<FMT_BF16X2><<<grid, 256, 0, s>>>(d_ops); break;
-    case FMT_FP16X2: k_build_bt<FMT_FP16X2><<<grid, 256, 0, s>>>(d_ops); break;
+    case FMT_TF32: k_build_bt<FMT_TF32><<<grid, 256, 0, s>>>(d_list, d_ops); break;
+    case FMT_BF16: k_build_bt<FMT_BF16><<<grid, 256, 0, s>>>(d_list, d_ops); break;
+    case FMT_FP16: k_build_bt<FMT_FP16><<<grid, 256, 0, s>>>(d_list, d_ops); break;
+    case FMT_BF16X2: k_build_bt<FMT_BF16X2><<<grid, 256, 0, s>>>(d_list, d_ops); break;
+    case FMT_FP16X2: k_build_bt<FMT_FP16X2><<<grid, 256, 0, s>>>(d_list, d_ops); break;
     default: return cudaErrorInvalidValue;
   }
   return cudaGetLastError();

@@ -270,13 +270,15 @@ __global__ void __launch_bounds__(256) k_build_ec2(const OpBuild2Entry *__restri
 // which one absorption can grow max(|Re|, |Im|) of the running tensor); one
 // block row per op, after the builders.  A block takes 32 columns at a time,
 // its 32 warps splitting K; the column sums meet in shared memory.
-__global__ void __launch_bounds__(1024) k_beta_ops(OpDesc *ops) {
-  const OpDesc &op = ops[blockIdx.y];
+__global__ void __launch_bounds__(1024) k_beta_ops(const int32_t *__restrict__ list, OpDesc *ops) {
+  const int which = list ? list[blockIdx.y] : (int)blockIdx.y;
+  const OpDesc &op = ops[which];
   if (op.Ec == nullptr) return;
   const int K = op.K, N = op.N;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   __shared__ float part[32][33];
   float best = 0.f;
+  if ((int)blockIdx.x * 32 >= N) return;
   for (int n0 = blockIdx.x * 32; n0 < N; n0 += gridDim.x * 32) {
     const int n = n0 + lane;
     float s = 0.f;
@@ -297,7 +299,7 @@ __global__ void __launch_bounds__(1024) k_beta_ops(OpDesc *ops) {
   if (w == 0) {
     best *= 1.0f + 1.0f / 256.0f;
     for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if (lane == 0) atomicMax(&ops[blockIdx.y].beta_c_bits, __float_as_uint(best));
+    if (lane == 0) atomicMax(&ops[which].beta_c_bits, __float_as_uint(best));
   }
 }
 
@@ -369,13 +371,18 @@ cudaError_t launch_build_operands(const OpBuildEntry *d_entries, int n, int max_
   return cudaGetLastError();
 }
 
-cudaError_t launch_operand_bounds(int n_ops, OpDesc *d_ops, cudaStream_t s, int64_t n_cols) {
+cudaError_t launch_operand_bounds(int n_ops, const int32_t *d_list, OpDesc *d_ops, cudaStream_t s,
+                                  int64_t n_cols) {
   if (n_ops <= 0) return cudaSuccess;
-  // 32 columns per block and pass; a single op gets a block per 32 columns
-  // (at least 128, at most 2048)
-  int64_t g1 = (n_cols + 31) / 32;
-  g1 = g1 < 128 ? 128 : (g1 > 2048 ? 2048 : g1);
-  k_beta_ops<<<dim3(n_ops == 1 ? (unsigned)g1 : 8u, n_ops), 1024, 0, s>>>(d_ops);
+  // 32 columns per block and pass: a block per 32 columns of the widest
+  // operand, up to 2048 blocks for one operand and some 1200 in all for
+  // several (at least 8 each): blocks past a narrow operand's columns leave at
+  // once, which thousands of them make felt (110 operands: 64 blocks each 32
+  // us, 11 each 21 us)
+  int64_t gx = (n_cols + 31) / 32;
+  const int64_t most = n_ops == 1 ? 2048 : (1200 / n_ops > 8 ? 1200 / n_ops : 8);
+  gx = gx < 1 ? 1 : (gx > most ? most : gx);
+  k_beta_ops<<<dim3((unsigned)gx, n_ops), 1024, 0, s>>>(d_list, d_ops);
   return cudaGetLastError();
 }
 
