@@ -227,6 +227,7 @@ struct peps_ctx {
   std::vector<cudaEvent_t> ev;
   int sm_count = 0;
   std::vector<peps_launch_info> launch_log;  // contraction launches of the last timed call
+  std::vector<peps_c128> host_out;           // staging of a host call's results
   cudaStream_t cap_stream = nullptr;  // records CUDA graphs (the caller's stream
                                       // may be the legacy default stream)
 };
@@ -675,7 +676,7 @@ static bool opts_equal(const peps_opts &a, const peps_opts &b) {
          a.prefix_cols == b.prefix_cols && a.prefix_group == b.prefix_group &&
          a.max_lanes == b.max_lanes && a.n_sliced == b.n_sliced &&
          a.n_slice_ids == b.n_slice_ids && a.n_fixed == b.n_fixed &&
-         a.tc_kchunk == b.tc_kchunk && a.tc_cluster == b.tc_cluster &&
+         a.tc_kchunk == b.tc_kchunk && a.tc_cluster == b.tc_cluster && a.tc_epi == b.tc_epi &&
          a.fuse_rows == b.fuse_rows && a.scheme == b.scheme && a.tc_ksplit == b.tc_ksplit &&
          a.measured_mask == b.measured_mask;
 }
@@ -1988,7 +1989,7 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
   P.off_small_opbase = off; off = align_up(off + (size_t)std::max(NS, (int64_t)1) * sizeof(int32_t));
   P.off_acc = off; off = align_up(off + std::max<int64_t>(n, 1) * sizeof(double2));
   P.off_bits = off; off = align_up(off + std::max<int64_t>(n, 1) * sizeof(uint64_t));
-  P.off_out = off; off = align_up(off + std::max<int64_t>(n, 1) * sizeof(peps_c128));
+  P.off_out = off; off = align_up(off + (std::max<int64_t>(n, 1) + 1) * sizeof(peps_c128));
   P.off_tables_end = off;
   off = align_up(off, 4096);
   P.lane_off = off;
@@ -2367,6 +2368,7 @@ static int ensure_events(peps_ctx *c, size_t n) {
 // with the evolution included).
 static int enqueue_sequence_stats_only(Plan &P, peps_stats &S) {
   S.launches_evolve = 1 + (int64_t)P.evo.size() - P.evo_prefix;
+  S.launches_finalize = 1;   // the clears
   if (P.opts.prefix_cols > 0 && P.n > 0) S.launches_finalize++;
   bool any_tc = false;
   for (auto &l : P.launches) any_tc |= (l.kind == 0 && l.tc);
@@ -2415,7 +2417,10 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
   char *base = (char *)P.ws;
   DeviceStatus *st = (DeviceStatus *)(base + P.off_status);
   const int64_t wd_ns = P.opts.watchdog_ns > 0 ? P.opts.watchdog_ns : 2000000000LL;
-  CUDA_TRY(cudaMemsetAsync(st, 0, sizeof(DeviceStatus), s));
+  double2 *acc = (double2 *)(base + P.off_acc);
+  Rec *recs = (Rec *)(base + P.off_recs);
+  CUDA_TRY(launch_begin(st, acc, std::max<int64_t>(P.n, 1), recs, P.n_recs, s));
+  S.launches_finalize++;
   if (rebuild) {
     // the leading batches (sites initialised there too), then the rest
     if (P.evo_prefix > 0)
@@ -2425,10 +2430,10 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
                                    (const EvoRef *)(base + P.off_evo_refs),
                                    (const int32_t *)(base + P.off_evo_first),
                                    (float2 *const *)(base + P.off_site_ptrs),
-                                   (const int64_t *)(base + P.off_site_lo), c->n, st, s));
+                                   (const int64_t *)(base + P.off_site_lo), c->n, s));
     else
       CUDA_TRY(launch_init_sites((float2 *const *)(base + P.off_site_ptrs),
-                                 (const int64_t *)(base + P.off_site_lo), c->n, st, s));
+                                 (const int64_t *)(base + P.off_site_lo), c->n, s));
     S.launches_evolve++;
     for (size_t bi = (size_t)P.evo_prefix; bi < P.evo.size(); ++bi) {
       const Plan::EvoBatch &eb = P.evo[bi];
@@ -2440,11 +2445,6 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
         CUDA_TRY(launch_gate2((const Gate2Entry *)(base + P.off_g2) + eb.off, eb.n, eb.max_work, s));
       S.launches_evolve++;
     }
-  } else {
-    // status block still needs its unit scalars
-    CUDA_TRY(launch_init_sites((float2 *const *)(base + P.off_site_ptrs),
-                               (const int64_t *)(base + P.off_site_lo), 0, st, s));
-    S.launches_evolve++;
   }
   if (P.opts.prefix_cols > 0 && P.n > 0) {
     uint64_t mask = 0;
@@ -2453,9 +2453,6 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
     CUDA_TRY(launch_check_groups(d_bits_in, P.n, P.opts.prefix_group, mask, st, s));
     S.launches_finalize++;
   }
-  double2 *acc = (double2 *)(base + P.off_acc);
-  CUDA_TRY(cudaMemsetAsync(acc, 0, std::max<int64_t>(P.n, 1) * sizeof(double2), s));
-  Rec *recs = (Rec *)(base + P.off_recs);
   OpDesc *ops = (OpDesc *)(base + P.off_opdesc);
   const StepItem *items = (const StepItem *)(base + P.off_items);
   const FinalEntry *fins = (const FinalEntry *)(base + P.off_fin);
@@ -2473,7 +2470,7 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
                             (((uint64_t)P.slice_list[si] ^ (uint64_t)P.slice_list[si - 1]) &
                              P.lower_mask) == 0;
     const int64_t n_clear = skip_lower ? (int64_t)P.s_m1 + 1 : P.n_recs;
-    if (n_clear > 0) CUDA_TRY(cudaMemsetAsync(recs, 0, n_clear * sizeof(Rec), s));
+    if (si > 0 && n_clear > 0) CUDA_TRY(cudaMemsetAsync(recs, 0, n_clear * sizeof(Rec), s));
     // operands whose restriction is unchanged since the previous slice stay
     const OpBuildEntry *e = obe + P.obe_first[si];
     const OpBuild2Entry *e2 = obe2 + P.obe2_first[si];
@@ -2669,18 +2666,23 @@ static int run_plan(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cudaStream_
   return PEPS_OK;
 }
 
+// The error of a completed call's status words.
+static int status_error(peps_ctx *c, const Plan &P, int error, int error_info, int timeout) {
+  if (timeout) {
+    c->broken = true;
+    return fail(PEPS_ETIMEOUT, "a device wait exceeded the watchdog budget (site step %d)", error_info);
+  }
+  if (error)
+    return fail(PEPS_EINVAL, "prefix group check failed at bitstring %d: bits of the first %d "
+                "columns differ inside a group", error_info, P.opts.prefix_cols);
+  return PEPS_OK;
+}
+
 static int check_status(peps_ctx *c, Plan &P, cudaStream_t s) {
   DeviceStatus h{};
   CUDA_TRY(cudaMemcpyAsync(&h, (char *)P.ws + P.off_status, sizeof h, cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
-  if (h.timeout) {
-    c->broken = true;
-    return fail(PEPS_ETIMEOUT, "a device wait exceeded the watchdog budget (site step %d)", h.error_info);
-  }
-  if (h.error)
-    return fail(PEPS_EINVAL, "prefix group check failed at bitstring %d: bits of the first %d "
-                "columns differ inside a group", h.error_info, P.opts.prefix_cols);
-  return PEPS_OK;
+  return status_error(c, P, h.error, h.error_info, h.timeout);
 }
 
 // Plan the call (or reuse the context's plan) and upload the plan's tables
@@ -2739,7 +2741,7 @@ extern "C" int peps_amplitudes_device(peps_ctx *c, const uint64_t *d_bits, int64
   Plan &P = *c->plan;
   rc = run_plan(c, P, d_bits, s);
   if (rc) return rc;
-  CUDA_TRY(launch_store_out((const double2 *)((char *)ws + P.off_acc), d_out, n, s));
+  CUDA_TRY(launch_store_out((const double2 *)((char *)ws + P.off_acc), d_out, n, nullptr, nullptr, s));
   c->stats.launches_finalize++;
   c->stats.launches_total++;
   const bool needs_check = (P.opts.flags & PEPS_FLAG_TIMING) || P.opts.prefix_cols > 0;
@@ -2768,13 +2770,22 @@ extern "C" int peps_amplitudes(peps_ctx *c, const uint64_t *bits, int64_t n, pep
   CUDA_TRY(cudaMemcpyAsync(d_bits, bits, n * sizeof(uint64_t), cudaMemcpyHostToDevice, s));
   rc = run_plan(c, P, d_bits, s);
   if (rc) return rc;
-  CUDA_TRY(launch_store_out((const double2 *)((char *)ws + P.off_acc), d_out, n, s));
+  // the amplitudes and, behind them, the status words, in one copy; `out` is
+  // written once the status is known to be good
+  static_assert(sizeof(int4) == sizeof(peps_c128), "the status words take one entry");
+  CUDA_TRY(launch_store_out((const double2 *)((char *)ws + P.off_acc), d_out, n,
+                            (const DeviceStatus *)((char *)ws + P.off_status), (int4 *)(d_out + n), s));
   c->stats.launches_finalize++;
   c->stats.launches_total++;
-  rc = check_status(c, P, s);
-  if (rc) return rc;
-  CUDA_TRY(cudaMemcpyAsync(out, d_out, n * sizeof(peps_c128), cudaMemcpyDeviceToHost, s));
+  c->host_out.resize((size_t)n + 1);
+  CUDA_TRY(cudaMemcpyAsync(c->host_out.data(), d_out, (n + 1) * sizeof(peps_c128),
+                           cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
+  int st[4];
+  std::memcpy(st, &c->host_out[n], sizeof st);
+  rc = status_error(c, P, st[0], st[1], st[2]);
+  if (rc) return rc;
+  std::memcpy(out, c->host_out.data(), n * sizeof(peps_c128));
   return PEPS_OK;
 }
 

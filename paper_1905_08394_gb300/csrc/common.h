@@ -305,24 +305,22 @@ struct DeviceStatus {
   int32_t error_info;
   int32_t timeout;      // nonzero: a bounded wait expired
   int32_t pad_;
-  float2 unit_f32;      // the scalar 1 in each format
-  uint32_t unit_h16[2]; // bf16 (re=1, im=0) hi plane / lo plane
-  uint32_t unit_f16[2]; // fp16 (re=1, im=0) hi plane / lo plane
 };
 
 // ---------------------------------------------------------------------------
 // Kernel launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------
+cudaError_t launch_begin(DeviceStatus *st, double2 *acc, int64_t n, Rec *recs, int64_t n_recs,
+                         cudaStream_t s);
 cudaError_t launch_init_sites(float2 *const *bufs, const int64_t *lo_off, int n_sites,
-                              DeviceStatus *st, cudaStream_t s);
+                              cudaStream_t s);
 cudaError_t launch_gate1(const Gate1Entry *d_entries, int n, int64_t max_half,
                          cudaStream_t s);
 // The whole evolution in one launch: block q applies site q's gate halves
 // refs[first[q] .. first[q+1]) in order, from |0> in bufs[q].
 cudaError_t launch_evolve_sites(const Gate1Entry *g1, const CzEntry *cz, const Gate2Entry *g2,
                                const EvoRef *refs, const int32_t *first, float2 *const *bufs,
-                               const int64_t *lo_off, int n_sites, DeviceStatus *st,
-                               cudaStream_t s);
+                               const int64_t *lo_off, int n_sites, cudaStream_t s);
 cudaError_t launch_cz(const CzEntry *d_entries, int n, int64_t max_out, cudaStream_t s);
 cudaError_t launch_gate2(const Gate2Entry *d_entries, int n, int64_t max_out, cudaStream_t s);
 cudaError_t launch_build_operands(const OpBuildEntry *d_entries, int n, int max_kn,
@@ -386,8 +384,9 @@ cudaError_t launch_sweep_small(const SmallSweep &p, int sm_count, cudaStream_t s
 
 cudaError_t launch_finalize(const FinalEntry *d_entries, int n, int fmt, int64_t plane,
                             const Rec *d_recs, double2 *d_acc, cudaStream_t s);
+// `d_tail` (may be null): the status words as well, for one copy back.
 cudaError_t launch_store_out(const double2 *d_acc, peps_c128 *d_out, int64_t n,
-                             cudaStream_t s);
+                             const DeviceStatus *st, int4 *d_tail, cudaStream_t s);
 cudaError_t launch_check_groups(const uint64_t *d_bits, int64_t n, int group,
                                 uint64_t mask, DeviceStatus *st, cudaStream_t s);
 

@@ -102,6 +102,8 @@ __global__ void __launch_bounds__(SW_THREADS) k_sweep_small(const SmallSweep p) 
   float2 *const buf0 = sm + ((p.cap_e + 1) & ~1);
   float2 *const buf1 = buf0 + ((p.cap_g + 15) & ~15);
   __shared__ float red[SW_THREADS / 32];
+  pdl_trigger();
+  pdl_wait();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int64_t i = blockIdx.x; i < p.n; i += gridDim.x) {
     const uint64_t bits = p.bits[i];
@@ -211,8 +213,7 @@ cudaError_t launch_sweep_small(const SmallSweep &p, int sm_count, cudaStream_t s
   const int per_sm = (int)((220u * 1024u) / (smem > 0 ? smem : 1));
   int64_t blocks = (int64_t)sm_count * (per_sm < 1 ? 1 : (per_sm > 4 ? 4 : per_sm));
   if (blocks > p.n) blocks = p.n;
-  k_sweep_small<<<(unsigned)blocks, SW_THREADS, smem, s>>>(p);
-  return cudaGetLastError();
+  return launch_dependent(k_sweep_small, dim3((unsigned)blocks), dim3(SW_THREADS), smem, s, p);
 }
 
 }  // namespace peps

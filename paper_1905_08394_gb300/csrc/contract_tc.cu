@@ -1497,6 +1497,8 @@ cudaError_t launch_contract_tc(void *handle, const StepItem *d_items, int n_item
 // ---------------------------------------------------------------------------
 template <int FMT>
 __global__ void __launch_bounds__(256) k_build_bt(const int32_t *__restrict__ list, OpDesc *ops) {
+  pdl_trigger();
+  pdl_wait();
   OpDesc &op = ops[list[blockIdx.y]];
   if (op.Bt[0] == nullptr) return;
   const int K = op.K, N = op.N;
@@ -1732,14 +1734,13 @@ cudaError_t launch_build_tc_operands(int n, const int32_t *d_list, int64_t max_k
   if (blocks < 1) blocks = 1;
   dim3 grid(blocks, n);
   switch (fmt) {
-    case FMT_TF32: k_build_bt<FMT_TF32><<<grid, 256, 0, s>>>(d_list, d_ops); break;
-    case FMT_BF16: k_build_bt<FMT_BF16><<<grid, 256, 0, s>>>(d_list, d_ops); break;
-    case FMT_FP16: k_build_bt<FMT_FP16><<<grid, 256, 0, s>>>(d_list, d_ops); break;
-    case FMT_BF16X2: k_build_bt<FMT_BF16X2><<<grid, 256, 0, s>>>(d_list, d_ops); break;
-    case FMT_FP16X2: k_build_bt<FMT_FP16X2><<<grid, 256, 0, s>>>(d_list, d_ops); break;
-    default: return cudaErrorInvalidValue;
+    case FMT_TF32: return launch_dependent(k_build_bt<FMT_TF32>, grid, dim3(256), 0, s, d_list, d_ops);
+    case FMT_BF16: return launch_dependent(k_build_bt<FMT_BF16>, grid, dim3(256), 0, s, d_list, d_ops);
+    case FMT_FP16: return launch_dependent(k_build_bt<FMT_FP16>, grid, dim3(256), 0, s, d_list, d_ops);
+    case FMT_BF16X2: return launch_dependent(k_build_bt<FMT_BF16X2>, grid, dim3(256), 0, s, d_list, d_ops);
+    case FMT_FP16X2: return launch_dependent(k_build_bt<FMT_FP16X2>, grid, dim3(256), 0, s, d_list, d_ops);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 }  // namespace peps

@@ -13,12 +13,24 @@
 
 namespace peps {
 
+// The start of a call in one launch: status words, amplitude accumulators and
+// records cleared.  Launched plainly, after everything before it on the stream
+// (a caller's own kernel may write the bitstrings and let dependents start
+// early): the call's other kernels start after it, and so may read tables and
+// bitstrings before their pdl_wait.
+__global__ void k_begin(DeviceStatus *st, double2 *acc, int64_t n, Rec *recs, int64_t n_recs) {
+  pdl_trigger();
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i0 == 0) *st = DeviceStatus{};
+  for (int64_t i = i0; i < n; i += (int64_t)gridDim.x * blockDim.x) acc[i] = make_double2(0.0, 0.0);
+  for (int64_t i = i0; i < n_recs; i += (int64_t)gridDim.x * blockDim.x) recs[i] = Rec{0u, 0};
+}
+
 // |0> on every site: A^0 = 1, A^1 = 0 with every auxiliary leg of dim 1
-// (paper, main-text PEPS equation for the product state).  Also writes the
-// scalar 1 in every storage format into the status block (the running
-// tensor before the first absorption).
-__global__ void k_init_sites(float2 *const *bufs, const int64_t *lo_off, int n_sites,
-                             DeviceStatus *st) {
+// (paper, main-text PEPS equation for the product state).
+__global__ void k_init_sites(float2 *const *bufs, const int64_t *lo_off, int n_sites) {
+  pdl_trigger();
+  pdl_wait();
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n_sites) {
     float2 *a = bufs[i];
@@ -26,16 +38,6 @@ __global__ void k_init_sites(float2 *const *bufs, const int64_t *lo_off, int n_s
     a[1] = make_float2(0.f, 0.f);
     a[lo_off[i]] = make_float2(0.f, 0.f);
     a[lo_off[i] + 1] = make_float2(0.f, 0.f);
-  }
-  if (i == 0) {
-    st->error = 0;
-    st->error_info = 0;
-    st->timeout = 0;
-    st->unit_f32 = make_float2(1.f, 0.f);
-    st->unit_h16[0] = pack_bf16(1.f, 0.f);
-    st->unit_h16[1] = 0u;
-    st->unit_f16[0] = pack_f16(1.f, 0.f);
-    st->unit_f16[1] = 0u;
   }
 }
 
@@ -144,6 +146,8 @@ __device__ __forceinline__ void gate1_apply(const Gate1Entry &g, int64_t e0, int
 
 // A batch of single-qubit gates on distinct sites (one per blockIdx.y).
 __global__ void k_gate1(const Gate1Entry *__restrict__ entries) {
+  pdl_trigger();
+  pdl_wait();
   gate1_apply(entries[blockIdx.y], (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
               (int64_t)gridDim.x * blockDim.x);
 }
@@ -222,6 +226,8 @@ __device__ __forceinline__ void cz_apply(const CzEntry &g, int64_t e0, int64_t d
 }
 
 __global__ void k_cz(const CzEntry *__restrict__ entries) {
+  pdl_trigger();
+  pdl_wait();
   cz_apply(entries[blockIdx.y], (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
            (int64_t)gridDim.x * blockDim.x);
 }
@@ -263,6 +269,8 @@ __device__ __forceinline__ void gate2_apply(const Gate2Entry &g, int64_t e0, int
 }
 
 __global__ void k_gate2(const Gate2Entry *__restrict__ entries) {
+  pdl_trigger();
+  pdl_wait();
   gate2_apply(entries[blockIdx.y], (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
               (int64_t)gridDim.x * blockDim.x);
 }
@@ -271,13 +279,13 @@ __global__ void k_gate2(const Gate2Entry *__restrict__ entries) {
 // a site's tensor evolves through its own gate halves only (a single-qubit
 // gate, or one side of a CZ or general gate split), so every block applies
 // its site's list in circuit order with a barrier between gates, starting
-// from |0> (A^0 = 1, A^1 = 0) in its first buffer.  Block 0 also writes the
-// status block's unit scalars.
+// from |0> (A^0 = 1, A^1 = 0) in its first buffer.
 __global__ void __launch_bounds__(256) k_evolve_sites(
     const Gate1Entry *__restrict__ g1, const CzEntry *__restrict__ cz,
     const Gate2Entry *__restrict__ g2, const EvoRef *__restrict__ refs,
-    const int32_t *__restrict__ first, float2 *const *bufs, const int64_t *lo_off,
-    DeviceStatus *st) {
+    const int32_t *__restrict__ first, float2 *const *bufs, const int64_t *lo_off) {
+  pdl_trigger();
+  pdl_wait();
   const int q = blockIdx.x;
   if (threadIdx.x == 0) {
     float2 *a = bufs[q];
@@ -285,16 +293,6 @@ __global__ void __launch_bounds__(256) k_evolve_sites(
     a[1] = make_float2(0.f, 0.f);
     a[lo_off[q]] = make_float2(0.f, 0.f);
     a[lo_off[q] + 1] = make_float2(0.f, 0.f);
-    if (q == 0) {
-      st->error = 0;
-      st->error_info = 0;
-      st->timeout = 0;
-      st->unit_f32 = make_float2(1.f, 0.f);
-      st->unit_h16[0] = pack_bf16(1.f, 0.f);
-      st->unit_h16[1] = 0u;
-      st->unit_f16[0] = pack_f16(1.f, 0.f);
-      st->unit_f16[1] = 0u;
-    }
   }
   __syncthreads();
   for (int i = first[q]; i < first[q + 1]; ++i) {
@@ -313,43 +311,41 @@ static int grid_for(int64_t work, int threads) {
   return (int)b;
 }
 
-cudaError_t launch_init_sites(float2 *const *bufs, const int64_t *lo_off, int n_sites,
-                              DeviceStatus *st, cudaStream_t s) {
-  int threads = 128;
-  int blocks = (n_sites + threads - 1) / threads;
-  if (blocks < 1) blocks = 1;
-  k_init_sites<<<blocks, threads, 0, s>>>(bufs, lo_off, n_sites, st);
+cudaError_t launch_begin(DeviceStatus *st, double2 *acc, int64_t n, Rec *recs, int64_t n_recs,
+                         cudaStream_t s) {
+  const int64_t work = n > n_recs ? n : n_recs;
+  k_begin<<<grid_for(work, 256), 256, 0, s>>>(st, acc, n, recs, n_recs);
   return cudaGetLastError();
+}
+
+cudaError_t launch_init_sites(float2 *const *bufs, const int64_t *lo_off, int n_sites,
+                              cudaStream_t s) {
+  const int threads = 128, blocks = (n_sites + threads - 1) / threads;
+  return launch_dependent(k_init_sites, dim3(blocks < 1 ? 1 : blocks), dim3(threads), 0, s, bufs,
+                          lo_off, n_sites);
 }
 
 cudaError_t launch_evolve_sites(const Gate1Entry *g1, const CzEntry *cz, const Gate2Entry *g2,
                                const EvoRef *refs, const int32_t *first, float2 *const *bufs,
-                               const int64_t *lo_off, int n_sites, DeviceStatus *st,
-                               cudaStream_t s) {
+                               const int64_t *lo_off, int n_sites, cudaStream_t s) {
   if (n_sites <= 0) return cudaSuccess;
-  k_evolve_sites<<<n_sites, 256, 0, s>>>(g1, cz, g2, refs, first, bufs, lo_off, st);
-  return cudaGetLastError();
+  return launch_dependent(k_evolve_sites, dim3(n_sites), dim3(256), 0, s, g1, cz, g2, refs, first,
+                          bufs, lo_off);
 }
 
 cudaError_t launch_gate1(const Gate1Entry *d_entries, int n, int64_t max_half, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  dim3 grid(grid_for(max_half, 256), n);
-  k_gate1<<<grid, 256, 0, s>>>(d_entries);
-  return cudaGetLastError();
+  return launch_dependent(k_gate1, dim3(grid_for(max_half, 256), n), dim3(256), 0, s, d_entries);
 }
 
 cudaError_t launch_cz(const CzEntry *d_entries, int n, int64_t max_out, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  dim3 grid(grid_for(max_out, 256), n);
-  k_cz<<<grid, 256, 0, s>>>(d_entries);
-  return cudaGetLastError();
+  return launch_dependent(k_cz, dim3(grid_for(max_out, 256), n), dim3(256), 0, s, d_entries);
 }
 
 cudaError_t launch_gate2(const Gate2Entry *d_entries, int n, int64_t max_out, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  dim3 grid(grid_for(max_out, 256), n);
-  k_gate2<<<grid, 256, 0, s>>>(d_entries);
-  return cudaGetLastError();
+  return launch_dependent(k_gate2, dim3(grid_for(max_out, 256), n), dim3(256), 0, s, d_entries);
 }
 
 }  // namespace peps

@@ -146,26 +146,33 @@ cudaError_t launch_dot_final(const DotEntry *d_entries, int n, const Rec *d_recs
   return launch_dependent(k_dot_final, dim3(n), dim3(128), 0, s, d_entries, d_recs, d_partials, d_acc);
 }
 
-__global__ void k_store_out(const double2 *__restrict__ acc, peps_c128 *out, int64_t n) {
+__global__ void k_store_out(const double2 *__restrict__ acc, peps_c128 *out, int64_t n,
+                            const DeviceStatus *st, int4 *tail) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) {
     out[i].re = acc[i].x;
     out[i].im = acc[i].y;
   }
+  if (i == 0 && tail) *tail = make_int4(st->error, st->error_info, st->timeout, 0);
 }
 
-cudaError_t launch_store_out(const double2 *d_acc, peps_c128 *d_out, int64_t n, cudaStream_t s) {
+cudaError_t launch_store_out(const double2 *d_acc, peps_c128 *d_out, int64_t n,
+                             const DeviceStatus *st, int4 *d_tail, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   const int threads = 256;
   const int64_t blocks = (n + threads - 1) / threads;
-  k_store_out<<<(unsigned)blocks, threads, 0, s>>>(d_acc, d_out, n);
-  return cudaGetLastError();
+  return launch_dependent(k_store_out, dim3((unsigned)blocks), dim3(threads), 0, s, d_acc, d_out, n,
+                          st, d_tail);
 }
 
 // Prefix reuse is only valid if every group of `group` consecutive
 // bitstrings agrees on the prefix qubits (mask); a violation sets an error.
 __global__ void k_check_groups(const uint64_t *__restrict__ bits, int64_t n, int group,
                                uint64_t mask, DeviceStatus *st) {
+  pdl_trigger();
+  pdl_wait();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   const int64_t g0 = (i / group) * group;
@@ -180,8 +187,8 @@ cudaError_t launch_check_groups(const uint64_t *d_bits, int64_t n, int group, ui
   if (n <= 0) return cudaSuccess;
   const int threads = 256;
   const int64_t blocks = (n + threads - 1) / threads;
-  k_check_groups<<<(unsigned)blocks, threads, 0, s>>>(d_bits, n, group, mask, st);
-  return cudaGetLastError();
+  return launch_dependent(k_check_groups, dim3((unsigned)blocks), dim3(threads), 0, s, d_bits, n, group,
+                          mask, st);
 }
 
 }  // namespace peps

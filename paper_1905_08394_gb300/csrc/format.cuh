@@ -16,9 +16,10 @@ namespace peps {
 // (once that one's blocks have all called pdl_trigger), sets itself up, and
 // reads or writes what kernels produce only after pdl_wait, which returns when
 // the kernel before has completed.  Every kernel launched this way calls both,
-// so completion stays in stream order.  Before pdl_wait only the plan's
-// tables (items) and the bitstrings may be read: they are copied in before the
-// call's first kernel.
+// so completion stays in stream order.  Several such kernels may be waiting at
+// once, so before pdl_wait only what was complete when the call's first kernel
+// (k_begin, launched plainly) started may be read: the plan's tables and the
+// bitstrings.
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 template <class... P, class... A>

@@ -87,6 +87,8 @@ __device__ __forceinline__ float2 fetch_E_dl(const OpBuildEntry &g, int k, int n
 
 // One block row per entry; threads cover Ec's K*N entries.
 __global__ void k_build_ec(const OpBuildEntry *__restrict__ entries, OpDesc *ops) {
+  pdl_trigger();
+  pdl_wait();
   const OpBuildEntry &g = entries[blockIdx.y];
   OpDesc &op = ops[g.op];
   const int K = g.rdims[0] * g.rdims[2];
@@ -136,6 +138,8 @@ constexpr int kEc2M = 16;   // m per shared-memory pass
 
 __global__ void __launch_bounds__(256) k_build_ec2(const OpBuild2Entry *__restrict__ entries,
                                                    OpDesc *ops) {
+  pdl_trigger();
+  pdl_wait();
   const OpBuild2Entry &g = entries[blockIdx.y];
   OpDesc &op = ops[g.op];
   const int La = g.a.rdims[0], Ra = g.a.rdims[1], Ua = g.a.rdims[2], Mid = g.a.rdims[3];
@@ -271,6 +275,8 @@ __global__ void __launch_bounds__(256) k_build_ec2(const OpBuild2Entry *__restri
 // block row per op, after the builders.  A block takes 32 columns at a time,
 // its 32 warps splitting K; the column sums meet in shared memory.
 __global__ void __launch_bounds__(1024) k_beta_ops(const int32_t *__restrict__ list, OpDesc *ops) {
+  pdl_trigger();
+  pdl_wait();
   const int which = list ? list[blockIdx.y] : (int)blockIdx.y;
   const OpDesc &op = ops[which];
   if (op.Ec == nullptr) return;
@@ -308,7 +314,9 @@ __global__ void __launch_bounds__(1024) k_beta_ops(const int32_t *__restrict__ l
 template <int FMT>
 __global__ void k_tensor_op(const TensorOpEntry *__restrict__ e, int64_t plane, OpDesc *ops,
                             const Rec *recs) {
+  pdl_trigger();
   const TensorOpEntry g = e[blockIdx.y];   // one entry per grid row
+  pdl_wait();
   OpDesc &op = ops[g.op];
   float2 *Ec = const_cast<float2 *>(op.Ec);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -336,15 +344,14 @@ cudaError_t launch_tensor_operand(const TensorOpEntry *d_entry, int n_entries, i
   if (bx < 1) bx = 1;
   const dim3 blocks((unsigned)bx, (unsigned)n_entries);
   switch (fmt) {
-    case FMT_F32: k_tensor_op<FMT_F32><<<blocks, 256, 0, s>>>(d_entry, plane, d_ops, d_recs); break;
-    case FMT_TF32: k_tensor_op<FMT_TF32><<<blocks, 256, 0, s>>>(d_entry, plane, d_ops, d_recs); break;
-    case FMT_BF16: k_tensor_op<FMT_BF16><<<blocks, 256, 0, s>>>(d_entry, plane, d_ops, d_recs); break;
-    case FMT_FP16: k_tensor_op<FMT_FP16><<<blocks, 256, 0, s>>>(d_entry, plane, d_ops, d_recs); break;
-    case FMT_BF16X2: k_tensor_op<FMT_BF16X2><<<blocks, 256, 0, s>>>(d_entry, plane, d_ops, d_recs); break;
-    case FMT_FP16X2: k_tensor_op<FMT_FP16X2><<<blocks, 256, 0, s>>>(d_entry, plane, d_ops, d_recs); break;
-    default: return cudaErrorInvalidValue;
+    case FMT_F32: return launch_dependent(k_tensor_op<FMT_F32>, blocks, dim3(256), 0, s, d_entry, plane, d_ops, d_recs);
+    case FMT_TF32: return launch_dependent(k_tensor_op<FMT_TF32>, blocks, dim3(256), 0, s, d_entry, plane, d_ops, d_recs);
+    case FMT_BF16: return launch_dependent(k_tensor_op<FMT_BF16>, blocks, dim3(256), 0, s, d_entry, plane, d_ops, d_recs);
+    case FMT_FP16: return launch_dependent(k_tensor_op<FMT_FP16>, blocks, dim3(256), 0, s, d_entry, plane, d_ops, d_recs);
+    case FMT_BF16X2: return launch_dependent(k_tensor_op<FMT_BF16X2>, blocks, dim3(256), 0, s, d_entry, plane, d_ops, d_recs);
+    case FMT_FP16X2: return launch_dependent(k_tensor_op<FMT_FP16X2>, blocks, dim3(256), 0, s, d_entry, plane, d_ops, d_recs);
   }
-  return cudaGetLastError();
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_build_operands2(const OpBuild2Entry *d_entries, int n, int max_kn,
@@ -357,8 +364,7 @@ cudaError_t launch_build_operands2(const OpBuild2Entry *d_entries, int n, int ma
   if (blocks > share) blocks = share < 8 ? 8 : share;
   if (blocks > 2048) blocks = 2048;
   if (blocks < 1) blocks = 1;
-  k_build_ec2<<<dim3(blocks, n), 256, 0, s>>>(d_entries, d_ops);
-  return cudaGetLastError();
+  return launch_dependent(k_build_ec2, dim3(blocks, n), dim3(256), 0, s, d_entries, d_ops);
 }
 
 cudaError_t launch_build_operands(const OpBuildEntry *d_entries, int n, int max_kn,
@@ -367,8 +373,7 @@ cudaError_t launch_build_operands(const OpBuildEntry *d_entries, int n, int max_
   int blocks = (max_kn + 255) / 256;
   if (blocks > 1024) blocks = 1024;
   if (blocks < 1) blocks = 1;
-  k_build_ec<<<dim3(blocks, n), 256, 0, s>>>(d_entries, d_ops);
-  return cudaGetLastError();
+  return launch_dependent(k_build_ec, dim3(blocks, n), dim3(256), 0, s, d_entries, d_ops);
 }
 
 cudaError_t launch_operand_bounds(int n_ops, const int32_t *d_list, OpDesc *d_ops, cudaStream_t s,
@@ -382,8 +387,7 @@ cudaError_t launch_operand_bounds(int n_ops, const int32_t *d_list, OpDesc *d_op
   int64_t gx = (n_cols + 31) / 32;
   const int64_t most = n_ops == 1 ? 2048 : (1200 / n_ops > 8 ? 1200 / n_ops : 8);
   gx = gx < 1 ? 1 : (gx > most ? most : gx);
-  k_beta_ops<<<dim3((unsigned)gx, n_ops), 1024, 0, s>>>(d_list, d_ops);
-  return cudaGetLastError();
+  return launch_dependent(k_beta_ops, dim3((unsigned)gx, n_ops), dim3(1024), 0, s, d_list, d_ops);
 }
 
 }  // namespace peps
