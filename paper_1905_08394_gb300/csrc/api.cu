@@ -168,9 +168,6 @@ struct Plan {
   // first slice builds every operand, a later one only those whose
   // restriction differs from the slice before it)
   std::vector<int64_t> obe_first, obe_count, obe2_first, obe2_count;
-  // the operands those builds write (bounds and planes follow for these only)
-  std::vector<int64_t> ol_first, ol_count;
-  size_t off_oplist = 0;
   int max_n_site = 1;           // widest site operand (N)
   int max_kn = 0;
   std::vector<int64_t> slice_list;
@@ -182,7 +179,8 @@ struct Plan {
   bool small = false;
   int small_cap_g = 0, small_cap_e = 0;
   size_t off_small_steps = 0, off_small_opbase = 0;
-  const uint64_t *small_bits = nullptr;
+  const uint64_t *call_bits = nullptr;
+  int n_opuse = 0;              // steps whose operands the call's start marks
   bool evo_sites = false;       // the whole evolution in one launch
   int evo_prefix = 0;           // leading gate batches done by that launch (a block
                                 // per site) while every site tensor is small; the
@@ -1614,8 +1612,6 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
   off = align_up(off + (size_t)std::max<int64_t>(n1, 1) * P.slice_list.size() * sizeof(OpBuildEntry));
   P.off_opbuild2 = off;
   off = align_up(off + (size_t)std::max<int64_t>(n2, 1) * P.slice_list.size() * sizeof(OpBuild2Entry));
-  P.off_oplist = off;
-  off = align_up(off + (size_t)std::max<int64_t>(n1 + n2, 1) * P.slice_list.size() * sizeof(int32_t));
 
   // records: chains = groups + bitstrings
   P.n_recs = (int)((P.n_groups + n) * P.n_steps);
@@ -1985,11 +1981,13 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
     }
     off = align_up(off + (quad ? per_lane * P.lanes * sizeof(double2) : 16));
   }
-  P.off_small_steps = off; off = align_up(off + (size_t)std::max(NS, (int64_t)1) * sizeof(SmallStep));
+  P.off_small_steps = off;
+  off = align_up(off + (size_t)std::max(NS, (int64_t)1) *
+                           (P.small ? sizeof(SmallStep) : sizeof(StepShape)));
   P.off_small_opbase = off; off = align_up(off + (size_t)std::max(NS, (int64_t)1) * sizeof(int32_t));
   P.off_acc = off; off = align_up(off + std::max<int64_t>(n, 1) * sizeof(double2));
   P.off_bits = off; off = align_up(off + std::max<int64_t>(n, 1) * sizeof(uint64_t));
-  P.off_out = off; off = align_up(off + (std::max<int64_t>(n, 1) + 1) * sizeof(peps_c128));
+  P.off_out = off; off = align_up(off + std::max<int64_t>(n, 1) * sizeof(peps_c128));
   P.off_tables_end = off;
   off = align_up(off, 4096);
   P.lane_off = off;
@@ -2005,7 +2003,7 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
   // ---- resolve addresses and assemble the table blob ----
   char *base = (char *)ws;
   const uint64_t *bsrc = host_bits ? (const uint64_t *)(base + P.off_bits) : bits_dev;
-  P.small_bits = bsrc;
+  P.call_bits = bsrc;
   for (size_t i = 0; i < items.size(); ++i) {
     items[i].bits = bsrc + rel[i].bit;
     items[i].A = rel[i].a_unit ? nullptr : (const void *)(base + P.lane_off + rel[i].a);
@@ -2059,9 +2057,24 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
       d.b_t = operand_scale_exp(fmt);
       d.K = sh.K;
       d.N = sh.N;
+      d.used = 1;
       ops[op] = d;
     }
   }
+  // A call of few lanes reads some of a step's operands (one bitstring one of
+  // four or eight, as do all members of a group in their shared part): the
+  // call's start marks them, and the builders make these only.  Many lanes
+  // read them all, and those of a small lattice are made in a few microseconds.
+  std::vector<OpUse> uses;
+  if (!P.small && n > 0 && n <= kMaxUseLanes)
+    for (int s = 0; s < P.n_steps; ++s) {
+      const StepShape &sh = P.steps[s];
+      if (sh.nq == 0) continue;
+      OpUse u{P.step_opbase[s], step_variants(sh), sh.q, sh.qs, sh.nq, sh.nx, {}};
+      for (int i = 0; i < sh.nx; ++i) u.xq[i] = sh.xq[i];
+      uses.push_back(u);
+    }
+  P.n_opuse = (int)uses.size();
   // operand build entries per slice: one per (step, variant)
   std::vector<OpBuildEntry> obe;
   std::vector<OpBuild2Entry> obe2;
@@ -2172,7 +2185,6 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
     }
   }
   // keep, for each slice after the first, only the entries that change
-  std::vector<int32_t> oplist;
   {
     const size_t n1 = (size_t)P.n_opbuild_per_slice, n2 = (size_t)P.n_obe2_per_slice;
     const size_t ns = P.slice_list.size();
@@ -2182,8 +2194,6 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
     P.obe_count.assign(ns, 0);
     P.obe2_first.assign(ns, 0);
     P.obe2_count.assign(ns, 0);
-    P.ol_first.assign(ns, 0);
-    P.ol_count.assign(ns, 0);
     for (size_t si = 0; si < ns; ++si) {
       P.obe_first[si] = (int64_t)c1.size();
       for (size_t j = 0; j < n1; ++j) {
@@ -2199,10 +2209,6 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
           c2.push_back(e);
       }
       P.obe2_count[si] = (int64_t)c2.size() - P.obe2_first[si];
-      P.ol_first[si] = (int64_t)oplist.size();
-      for (int64_t j = P.obe_first[si]; j < (int64_t)c1.size(); ++j) oplist.push_back(c1[j].op);
-      for (int64_t j = P.obe2_first[si]; j < (int64_t)c2.size(); ++j) oplist.push_back(c2[j].op);
-      P.ol_count[si] = (int64_t)oplist.size() - P.ol_first[si];
     }
     obe.swap(c1);
     obe2.swap(c2);
@@ -2230,12 +2236,14 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
     std::vector<SmallStep> ss;
     for (const auto &sh : P.steps) ss.push_back(small_step(sh));
     put(P.off_small_steps, ss.data(), ss.size() * sizeof(SmallStep));
+  } else {   // no step descriptions: their place holds the operand uses
+    static_assert(sizeof(OpUse) <= sizeof(StepShape), "a use fits a step's place");
+    put(P.off_small_steps, uses.data(), uses.size() * sizeof(OpUse));
   }
   put(P.off_small_opbase, P.step_opbase.data(), P.step_opbase.size() * sizeof(int32_t));
   put(P.off_opdesc, ops.data(), ops.size() * sizeof(OpDesc));
   put(P.off_opbuild, obe.data(), obe.size() * sizeof(OpBuildEntry));
   put(P.off_opbuild2, obe2.data(), obe2.size() * sizeof(OpBuild2Entry));
-  put(P.off_oplist, oplist.data(), oplist.size() * sizeof(int32_t));
   put(P.off_items, items.data(), items.size() * sizeof(StepItem));
   put(P.off_fin, fins.data(), fins.size() * sizeof(FinalEntry));
   put(P.off_tops, tops.data(), tops.size() * sizeof(TensorOpEntry));
@@ -2402,7 +2410,7 @@ static int enqueue_sequence_stats_only(Plan &P, peps_stats &S) {
   const int64_t ns = (int64_t)P.slice_list.size();
   for (int64_t si = 0; si < ns; ++si)
     S.launches_operand += (P.obe_count[si] > 0 ? 1 : 0) + (P.obe2_count[si] > 0 ? 1 : 0) +
-                          (P.ol_count[si] > 0 ? 1 + (any_tc ? 1 : 0) : 0);
+                          (P.obe_count[si] + P.obe2_count[si] > 0 ? 1 + (any_tc ? 1 : 0) : 0);
   const int64_t nl = lower_runs(P);
   for (auto &l : P.launches) {
     const int64_t k = l.lower ? nl : ns;
@@ -2446,7 +2454,9 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
   const int64_t wd_ns = P.opts.watchdog_ns > 0 ? P.opts.watchdog_ns : 2000000000LL;
   double2 *acc = (double2 *)(base + P.off_acc);
   Rec *recs = (Rec *)(base + P.off_recs);
-  CUDA_TRY(launch_begin(st, acc, std::max<int64_t>(P.n, 1), recs, P.n_recs, s));
+  CUDA_TRY(launch_begin(st, acc, std::max<int64_t>(P.n, 1), recs, P.n_recs,
+                        (const OpUse *)(base + P.off_small_steps), P.n_opuse, P.call_bits,
+                        (OpDesc *)(base + P.off_opdesc), s));
   S.launches_finalize++;
   if (rebuild) {
     // the leading batches (sites initialised there too), then the rest
@@ -2483,6 +2493,7 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
   OpDesc *ops = (OpDesc *)(base + P.off_opdesc);
   const StepItem *items = (const StepItem *)(base + P.off_items);
   const FinalEntry *fins = (const FinalEntry *)(base + P.off_fin);
+  const bool marked = P.n_opuse > 0;
   const OpBuildEntry *obe = (const OpBuildEntry *)(base + P.off_opbuild);
   const OpBuild2Entry *obe2 = (const OpBuild2Entry *)(base + P.off_opbuild2);
   const TensorOpEntry *tops = (const TensorOpEntry *)(base + P.off_tops);
@@ -2502,20 +2513,22 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
     const OpBuildEntry *e = obe + P.obe_first[si];
     const OpBuild2Entry *e2 = obe2 + P.obe2_first[si];
     if (P.obe_count[si] > 0) {
-      CUDA_TRY(launch_build_operands(e, (int)P.obe_count[si], P.max_kn, ops, s));
+      CUDA_TRY(launch_build_operands(e, (int)P.obe_count[si], P.max_kn, ops, marked, s));
       S.launches_operand++;
     }
     if (P.obe2_count[si] > 0) {
-      CUDA_TRY(launch_build_operands2(e2, (int)P.obe2_count[si], P.max_kn2, ops, s));
+      CUDA_TRY(launch_build_operands2(e2, (int)P.obe2_count[si], P.max_kn2, ops,
+                                      marked, c->sm_count, s));
       S.launches_operand++;
     }
-    const int32_t *ol = (const int32_t *)(base + P.off_oplist) + P.ol_first[si];
-    const int n_ol = (int)P.ol_count[si];
+    const OpList ol{e, e2, (int)P.obe_count[si]};
+    const int n_ol = (int)(P.obe_count[si] + P.obe2_count[si]);
     if (n_ol > 0) {
-      CUDA_TRY(launch_operand_bounds(n_ol, ol, ops, s, P.max_n_site));
+      CUDA_TRY(launch_operand_bounds(n_ol, ol, ops, s, P.max_n_site, marked, c->sm_count));
       S.launches_operand++;
       if (any_tc) {
-        CUDA_TRY(launch_build_tc_operands(n_ol, ol, std::max(P.max_kn, P.max_kn2), ops, P.fmt, s));
+        CUDA_TRY(launch_build_tc_operands(n_ol, ol, std::max(P.max_kn, P.max_kn2), ops, P.fmt, marked,
+                                          c->sm_count, s));
         S.launches_operand++;
       }
     }
@@ -2528,7 +2541,7 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
           sw.steps = (const SmallStep *)(base + P.off_small_steps);
           sw.op_base = (const int32_t *)(base + P.off_small_opbase);
           sw.ops = ops;
-          sw.bits = P.small_bits;
+          sw.bits = P.call_bits;
           sw.acc = acc;
           sw.n = P.n;
           sw.n_steps = P.n_steps;
@@ -2562,7 +2575,8 @@ static int enqueue_sequence(peps_ctx *c, Plan &P, const uint64_t *d_bits_in, cud
         } else {
           CUDA_TRY(launch_tensor_operand(tops + l.aux_off, l.n_aux, l.kn, P.fmt, P.plane, ops, recs,
                                          s));
-          CUDA_TRY(launch_operand_bounds(l.n_aux, nullptr, ops + l.op, s, l.shape.N));
+          CUDA_TRY(launch_operand_bounds(l.n_aux, OpList{}, ops + l.op, s, l.shape.N, false,
+                                         c->sm_count));
         }
         S.launches_operand += 2;
       } else if (l.kind == 3 && l.fused_merge >= 0) {
@@ -2788,22 +2802,23 @@ extern "C" int peps_amplitudes(peps_ctx *c, const uint64_t *bits, int64_t n, pep
   CUDA_TRY(cudaMemcpyAsync(d_bits, bits, n * sizeof(uint64_t), cudaMemcpyHostToDevice, s));
   rc = run_plan(c, P, d_bits, s);
   if (rc) return rc;
-  // the amplitudes and, behind them, the status words, in one copy; `out` is
-  // written once the status is known to be good
+  // the status words (over the end of the bitstrings, which every kernel has
+  // read by then) and the amplitudes in one copy; `out` is written once the
+  // status is known to be good
   static_assert(sizeof(int4) == sizeof(peps_c128), "the status words take one entry");
   CUDA_TRY(launch_store_out((const double2 *)((char *)ws + P.off_acc), d_out, n,
-                            (const DeviceStatus *)((char *)ws + P.off_status), (int4 *)(d_out + n), s));
+                            (const DeviceStatus *)((char *)ws + P.off_status), (int4 *)(d_out - 1), s));
   c->stats.launches_finalize++;
   c->stats.launches_total++;
   c->host_out.resize((size_t)n + 1);
-  CUDA_TRY(cudaMemcpyAsync(c->host_out.data(), d_out, (n + 1) * sizeof(peps_c128),
+  CUDA_TRY(cudaMemcpyAsync(c->host_out.data(), d_out - 1, (n + 1) * sizeof(peps_c128),
                            cudaMemcpyDeviceToHost, s));
   CUDA_TRY(cudaStreamSynchronize(s));
   int st[4];
-  std::memcpy(st, &c->host_out[n], sizeof st);
+  std::memcpy(st, &c->host_out[0], sizeof st);
   rc = status_error(c, P, st[0], st[1], st[2]);
   if (rc) return rc;
-  std::memcpy(out, c->host_out.data(), n * sizeof(peps_c128));
+  std::memcpy(out, c->host_out.data() + 1, n * sizeof(peps_c128));
   return PEPS_OK;
 }
 

@@ -85,7 +85,9 @@ struct OpDesc {
   const void *Bt[2];    // tensor-core planes [Nr_pad][Kr_pad] (hi, lo), or null
   uint32_t beta_c_bits; // max_n sum_k (|Re E_kn| + |Im E_kn|), float bits
   uint32_t beta_t_bits; // same bound for the scaled tensor-core planes
-  int32_t b_t;          // scale exponent of the tensor-core planes (Bt = Ec 2^b_t)
+  int16_t b_t;          // scale exponent of the tensor-core planes (Bt = Ec 2^b_t)
+  int16_t used;         // site operand: some lane of the call reads it (k_begin);
+                        // the builders pass over the others
   int32_t K, N;         // complex dims
   int32_t e_c;          // Ec = E 2^e_c (0 for site operands; a merge operand
                         // built from a stored tensor carries that tensor's scale)
@@ -165,7 +167,8 @@ struct StepShape {
 // Operand index of a lane for a block: bit j = output bit of the block's
 // j-th site (for one site: tau), then bit nq + i = output bit of qubit xq[i]
 // (the held bond bits of the block's legs that depend on a neighbour).
-__host__ __device__ inline int block_variant(uint64_t bits, const StepShape &sh) {
+template <class Step>   // StepShape, or what it needs of one
+__host__ __device__ inline int block_variant(uint64_t bits, const Step &sh) {
   int v = 0;
   for (int j = 0; j < sh.nq; ++j) v |= (int)((bits >> (sh.q + j * sh.qs)) & 1ull) << j;
   for (int i = 0; i < sh.nx; ++i) v |= (int)((bits >> sh.xq[i]) & 1ull) << (sh.nq + i);
@@ -174,6 +177,15 @@ __host__ __device__ inline int block_variant(uint64_t bits, const StepShape &sh)
 
 // Operand variants of a step.
 __host__ __device__ inline int step_variants(const StepShape &sh) { return 1 << (sh.nq + sh.nx); }
+
+// A step's site operands, for marking the ones that a call reads.
+struct OpUse {
+  int32_t op_base, n_var;    // its OpDescs: op_base .. op_base + n_var
+  int32_t q, qs, nq, nx;     // as in StepShape
+  int32_t xq[4];
+};
+// Most lanes for which a call marks them (above it every operand counts as read).
+constexpr int kMaxUseLanes = 1024;
 
 // Evolution tables.  Site tensors are kept as float-float pairs: a hi plane
 // and a lo plane (value = hi + lo), the lo plane `lo_off` entries after the
@@ -263,6 +275,17 @@ struct OpBuild2Entry {
   int32_t pad_;
 };
 
+// The operands of n1 one-site and further two-site build entries, in that
+// order; without entries, operand j is j.
+struct OpList {
+  const OpBuildEntry *e1;
+  const OpBuild2Entry *e2;
+  int32_t n1;
+  __device__ __forceinline__ int op(int j) const {
+    return !e1 ? j : j < n1 ? e1[j].op : e2[j - n1].op;
+  }
+};
+
 // Operand of a merge built from a finished quarter (or half) tensor G held in
 // the running-tensor format:  Ec[k][n] = G[k ks + n_hi ns_hi + n_lo ns] 2^-target
 // with n = n_hi * Nlo + n_lo (so that |Ec| <= 1), and e_c of the op =
@@ -311,6 +334,7 @@ struct DeviceStatus {
 // Kernel launchers (defined in the .cu files)
 // ---------------------------------------------------------------------------
 cudaError_t launch_begin(DeviceStatus *st, double2 *acc, int64_t n, Rec *recs, int64_t n_recs,
+                         const OpUse *uses, int n_uses, const uint64_t *bits, OpDesc *ops,
                          cudaStream_t s);
 cudaError_t launch_init_sites(float2 *const *bufs, const int64_t *lo_off, int n_sites,
                               cudaStream_t s);
@@ -323,12 +347,13 @@ cudaError_t launch_evolve_sites(const Gate1Entry *g1, const CzEntry *cz, const G
                                const int64_t *lo_off, int n_sites, cudaStream_t s);
 cudaError_t launch_cz(const CzEntry *d_entries, int n, int64_t max_out, cudaStream_t s);
 cudaError_t launch_gate2(const Gate2Entry *d_entries, int n, int64_t max_out, cudaStream_t s);
+// Site operands; `marked`: those that k_begin found unread are passed over.
 cudaError_t launch_build_operands(const OpBuildEntry *d_entries, int n, int max_kn,
-                                  OpDesc *d_ops, cudaStream_t s);
-// Bounds of the listed ops (d_list null: ops 0 .. n_ops - 1); `n_cols`: the
+                                  OpDesc *d_ops, bool marked, cudaStream_t s);
+// Bounds of the listed ops (without a list: ops 0 .. n_ops - 1); `n_cols`: the
 // widest operand's N.
-cudaError_t launch_operand_bounds(int n_ops, const int32_t *d_list, OpDesc *d_ops, cudaStream_t s,
-                                  int64_t n_cols);
+cudaError_t launch_operand_bounds(int n_ops, const OpList &list, OpDesc *d_ops, cudaStream_t s,
+                                  int64_t n_cols, bool marked, int sm_count);
 cudaError_t launch_tensor_operand(const TensorOpEntry *d_entries, int n_entries, int64_t kn,
                                   int fmt, int64_t plane, OpDesc *d_ops, const Rec *d_recs,
                                   cudaStream_t s);
@@ -340,15 +365,15 @@ cudaError_t launch_dot(const DotEntry *d_entries, int n, int fmt, int64_t plane,
 cudaError_t launch_dot_final(const DotEntry *d_entries, int n, const Rec *d_recs,
                              const double2 *d_partials, double2 *d_acc, cudaStream_t s);
 cudaError_t launch_build_operands2(const OpBuild2Entry *d_entries, int n, int max_kn,
-                                   OpDesc *d_ops, cudaStream_t s);
+                                   OpDesc *d_ops, bool marked, int sm_count, cudaStream_t s);
 // A merge operand's tensor-core planes and bound straight from the stored
 // tensor (no Ec); K, N are the operand's sizes.
 cudaError_t launch_tensor_operand_tc(const TensorOpEntry *d_entries, int n_entries, int K, int N,
                                      int fmt, int64_t plane, OpDesc *d_ops, const Rec *d_recs,
                                      cudaStream_t s);
 // Tensor-core planes (and their bound) of the listed ops from their Ec.
-cudaError_t launch_build_tc_operands(int n_ops, const int32_t *d_list, int64_t max_kn,
-                                     OpDesc *d_ops, int fmt, cudaStream_t s);
+cudaError_t launch_build_tc_operands(int n_ops, const OpList &list, int64_t max_kn,
+                                     OpDesc *d_ops, int fmt, bool marked, int sm_count, cudaStream_t s);
 cudaError_t launch_contract_simt(const StepShape &sh, const StepItem *d_items, int n_items,
                                  const OpDesc *d_ops, Rec *d_recs, const DeviceStatus *st,
                                  cudaStream_t s, bool aligned32);

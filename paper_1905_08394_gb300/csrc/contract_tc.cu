@@ -49,6 +49,7 @@
 
 #include "common.h"
 #include "format.cuh"
+#include "share.cuh"
 
 namespace peps {
 
@@ -1495,12 +1496,14 @@ cudaError_t launch_contract_tc(void *handle, const StepItem *d_items, int n_item
 // Tensor-core operand build: the real embedding of E (scaled by 2^b_t), split
 // into the form's planes, K-major [Nr][Kr].  Also the bound beta_t.
 // ---------------------------------------------------------------------------
+// Tiles first, first + step, ... below last of one operand: 32 x 32 entries of
+// Ec each, through shared memory.
+__device__ __forceinline__ int bt_tiles(const OpDesc &op, bool marked) {   // none if no lane reads it
+  if (op.Bt[0] == nullptr || (marked && !op.used)) return 0;
+  return ((op.K + 31) / 32) * ((op.N + 31) / 32);
+}
 template <int FMT>
-__global__ void __launch_bounds__(256) k_build_bt(const int32_t *__restrict__ list, OpDesc *ops) {
-  pdl_trigger();
-  pdl_wait();
-  OpDesc &op = ops[list[blockIdx.y]];
-  if (op.Bt[0] == nullptr) return;
+__device__ __forceinline__ void bt_operand_tiles(OpDesc &op, int first, int last, int step) {
   const int K = op.K, N = op.N;
   const float sc = ldexpf(1.f, op.b_t);
   const float2 *const Ec = op.Ec;
@@ -1508,9 +1511,9 @@ __global__ void __launch_bounds__(256) k_build_bt(const int32_t *__restrict__ li
   // 32 x 32 complex tiles of Ec through shared memory: read along n, written
   // along k, two real columns (a = 0, 1 of one k) per store
   __shared__ float2 tile[32][33];
-  const int tn = (N + 31) / 32, n_tiles = ((K + 31) / 32) * tn;
+  const int tn = (N + 31) / 32;
   const int64_t Kr = 2 * (int64_t)K;
-  for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+  for (int t = first; t < last; t += step) {
     const int k0 = (t / tn) * 32, n0 = (t % tn) * 32;
     for (int e = threadIdx.x; e < 32 * 32; e += blockDim.x) {
       const int kk = e >> 5, nn = e & 31;
@@ -1565,12 +1568,28 @@ __global__ void __launch_bounds__(256) k_build_bt(const int32_t *__restrict__ li
     }
     __syncthreads();
   }
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if (first == 0 && threadIdx.x == 0) {
     // beta_t = beta_c * 2^b_t (beta_c already carries a rounding margin; the
     // rounded planes differ from the scaled values by at most 2^-8 relative)
     const float bc = __uint_as_float(op.beta_c_bits);
     op.beta_t_bits = __float_as_uint(bc * sc * (1.0f + 1.0f / 128.0f));
   }
+}
+
+template <int FMT>
+__global__ void __launch_bounds__(256) k_build_bt(const OpList list, int n, OpDesc *ops,
+                                                  bool marked) {
+  pdl_trigger();
+  pdl_wait();
+  if (gridDim.y > 1 || n == 1) {   // by operand
+    OpDesc &op = ops[list.op(blockIdx.y)];
+    const int nt = bt_tiles(op, marked);
+    if ((int)blockIdx.x < nt) bt_operand_tiles<FMT>(op, blockIdx.x, nt, gridDim.x);
+    return;
+  }
+  auto tiles = [&](int j) { return bt_tiles(ops[list.op(j)], marked); };
+  for_block_share(n, (int)threadIdx.x < n ? tiles(threadIdx.x) : 0, tiles,
+                  [&](int j, int a, int b) { bt_operand_tiles<FMT>(ops[list.op(j)], a, b, 1); });
 }
 
 // A merge operand straight from a stored tensor G whose k index is contiguous:
@@ -1724,21 +1743,20 @@ cudaError_t launch_tensor_operand_tc(const TensorOpEntry *d_entry, int n_entries
   return cudaErrorInvalidValue;
 }
 
-cudaError_t launch_build_tc_operands(int n, const int32_t *d_list, int64_t max_kn, OpDesc *d_ops,
-                                     int fmt, cudaStream_t s) {
+cudaError_t launch_build_tc_operands(int n, const OpList &list, int64_t max_kn, OpDesc *d_ops,
+                                     int fmt, bool marked, int sm_count, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  // 32 x 32 tiles of the largest operand, up to 128 blocks each (blocks of
-  // smaller operands leave at once, which thousands of them make felt)
-  int64_t blocks = (max_kn + 1023) / 1024 + 2;
-  if (blocks > 128) blocks = 128;
-  if (blocks < 1) blocks = 1;
-  dim3 grid(blocks, n);
+  // the list of all operands' tiles, or by operand where that gives about
+  // every tile its own block
+  const int64_t tiles = (max_kn + 1023) / 1024 + 2;
+  const dim3 grid = n == 1 || n * tiles <= 2048 ? dim3((unsigned)(tiles < 2048 ? tiles : 2048), n)
+                                                : dim3(6 * sm_count);
   switch (fmt) {
-    case FMT_TF32: return launch_dependent(k_build_bt<FMT_TF32>, grid, dim3(256), 0, s, d_list, d_ops);
-    case FMT_BF16: return launch_dependent(k_build_bt<FMT_BF16>, grid, dim3(256), 0, s, d_list, d_ops);
-    case FMT_FP16: return launch_dependent(k_build_bt<FMT_FP16>, grid, dim3(256), 0, s, d_list, d_ops);
-    case FMT_BF16X2: return launch_dependent(k_build_bt<FMT_BF16X2>, grid, dim3(256), 0, s, d_list, d_ops);
-    case FMT_FP16X2: return launch_dependent(k_build_bt<FMT_FP16X2>, grid, dim3(256), 0, s, d_list, d_ops);
+    case FMT_TF32: return launch_dependent(k_build_bt<FMT_TF32>, grid, dim3(256), 0, s, list, n, d_ops, marked);
+    case FMT_BF16: return launch_dependent(k_build_bt<FMT_BF16>, grid, dim3(256), 0, s, list, n, d_ops, marked);
+    case FMT_FP16: return launch_dependent(k_build_bt<FMT_FP16>, grid, dim3(256), 0, s, list, n, d_ops, marked);
+    case FMT_BF16X2: return launch_dependent(k_build_bt<FMT_BF16X2>, grid, dim3(256), 0, s, list, n, d_ops, marked);
+    case FMT_FP16X2: return launch_dependent(k_build_bt<FMT_FP16X2>, grid, dim3(256), 0, s, list, n, d_ops, marked);
   }
   return cudaErrorInvalidValue;
 }

@@ -14,16 +14,30 @@
 namespace peps {
 
 // The start of a call in one launch: status words, amplitude accumulators and
-// records cleared.  Launched plainly, after everything before it on the stream
-// (a caller's own kernel may write the bitstrings and let dependents start
-// early): the call's other kernels start after it, and so may read tables and
-// bitstrings before their pdl_wait.
-__global__ void k_begin(DeviceStatus *st, double2 *acc, int64_t n, Rec *recs, int64_t n_recs) {
+// records cleared, and (a block per step behind the clearing ones) the site
+// operands marked that some lane's bitstring selects.  Launched plainly, after
+// everything before it on the stream (a caller's own kernel may write the
+// bitstrings and let dependents start early): the call's other kernels start
+// after it, and so may read tables and bitstrings before their pdl_wait.
+__global__ void k_begin(DeviceStatus *st, double2 *acc, int64_t n, Rec *recs, int64_t n_recs,
+                        const OpUse *__restrict__ uses, int n_uses,
+                        const uint64_t *__restrict__ bits, OpDesc *ops) {
   pdl_trigger();
+  const int n_clear = (int)gridDim.x - n_uses;
+  if ((int)blockIdx.x >= n_clear) {
+    const OpUse u = uses[blockIdx.x - n_clear];
+    for (int v = threadIdx.x; v < u.n_var; v += blockDim.x) ops[u.op_base + v].used = 0;
+    __syncthreads();
+#pragma unroll 4
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x)
+      ops[u.op_base + block_variant(bits[i], u)].used = 1;
+    return;
+  }
   const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t step = (int64_t)n_clear * blockDim.x;
   if (i0 == 0) *st = DeviceStatus{};
-  for (int64_t i = i0; i < n; i += (int64_t)gridDim.x * blockDim.x) acc[i] = make_double2(0.0, 0.0);
-  for (int64_t i = i0; i < n_recs; i += (int64_t)gridDim.x * blockDim.x) recs[i] = Rec{0u, 0};
+  for (int64_t i = i0; i < n; i += step) acc[i] = make_double2(0.0, 0.0);
+  for (int64_t i = i0; i < n_recs; i += step) recs[i] = Rec{0u, 0};
 }
 
 // |0> on every site: A^0 = 1, A^1 = 0 with every auxiliary leg of dim 1
@@ -312,9 +326,11 @@ static int grid_for(int64_t work, int threads) {
 }
 
 cudaError_t launch_begin(DeviceStatus *st, double2 *acc, int64_t n, Rec *recs, int64_t n_recs,
+                         const OpUse *uses, int n_uses, const uint64_t *bits, OpDesc *ops,
                          cudaStream_t s) {
   const int64_t work = n > n_recs ? n : n_recs;
-  k_begin<<<grid_for(work, 256), 256, 0, s>>>(st, acc, n, recs, n_recs);
+  k_begin<<<grid_for(work, 256) + n_uses, 256, 0, s>>>(st, acc, n, recs, n_recs, uses, n_uses,
+                                                       bits, ops);
   return cudaGetLastError();
 }
 

@@ -11,6 +11,7 @@
 // its single Schmidt term.  Only two operands exist per site and slice, so the
 // cost does not depend on the number of bitstrings.
 #include "common.h"
+#include "share.cuh"
 #include "format.cuh"
 
 namespace peps {
@@ -86,11 +87,12 @@ __device__ __forceinline__ float2 fetch_E_dl(const OpBuildEntry &g, int k, int n
 }
 
 // One block row per entry; threads cover Ec's K*N entries.
-__global__ void k_build_ec(const OpBuildEntry *__restrict__ entries, OpDesc *ops) {
+__global__ void k_build_ec(const OpBuildEntry *__restrict__ entries, OpDesc *ops, bool marked) {
   pdl_trigger();
   pdl_wait();
   const OpBuildEntry &g = entries[blockIdx.y];
   OpDesc &op = ops[g.op];
+  if (marked && !op.used) return;
   const int K = g.rdims[0] * g.rdims[2];
   const int N = g.rdims[1] * g.rdims[3];
   float2 *Ec = const_cast<float2 *>(op.Ec);
@@ -135,20 +137,24 @@ __device__ __forceinline__ void acc_prod(float x, float y, float &s, float &c) {
 // thread accumulates four entries (one column, four rows).
 constexpr int kEc2T = 32;   // tile rows and columns
 constexpr int kEc2M = 16;   // m per shared-memory pass
+constexpr int kEc2Blocks = 5;   // resident per SM (40 KB of shared memory each)
 
-__global__ void __launch_bounds__(256) k_build_ec2(const OpBuild2Entry *__restrict__ entries,
-                                                   OpDesc *ops) {
-  pdl_trigger();
-  pdl_wait();
-  const OpBuild2Entry &g = entries[blockIdx.y];
+// 32 x 32 tiles of an entry's product.
+__device__ __forceinline__ int ec2_tiles(const OpBuild2Entry &g) {
+  const int rows = g.a.rdims[0] * g.a.rdims[2] * g.a.rdims[1];
+  const int cols = g.b.rdims[0] * g.b.rdims[1] * g.b.rdims[3];
+  return ((rows + kEc2T - 1) / kEc2T) * ((cols + kEc2T - 1) / kEc2T);
+}
+
+// Tiles ta, ta + step, ... below tb of an entry.
+__device__ __forceinline__ void ec2_entry_tiles(const OpBuild2Entry &g, OpDesc *ops, int ta, int tb,
+                                                int step) {
   OpDesc &op = ops[g.op];
   const int La = g.a.rdims[0], Ra = g.a.rdims[1], Ua = g.a.rdims[2], Mid = g.a.rdims[3];
   const int Lb = g.b.rdims[0], Rb = g.b.rdims[1], Db = g.b.rdims[3];
   const int N = Ra * Rb * Db;
   const int Rows = La * Ua * Ra, Cols = Lb * Rb * Db;
   const int tiles_c = (Cols + kEc2T - 1) / kEc2T;
-  const int n_tiles = ((Rows + kEc2T - 1) / kEc2T) * tiles_c;
-  if ((int)blockIdx.x >= n_tiles) return;
   // full index of every restricted value of the shared bond, on both sites,
   // and (where the legs are short enough) element offsets of the other legs
   __shared__ int mid_a[kMaxMid], mid_b[kMaxMid];
@@ -157,27 +163,36 @@ __global__ void __launch_bounds__(256) k_build_ec2(const OpBuild2Entry *__restri
   __shared__ float4 As[kEc2T][kEc2M + 1];   // (hi re, hi im, lo re, lo im), padded rows
   __shared__ float4 Bs[kEc2M][kEc2T];
   __shared__ int64_t row_a[kEc2T], col_b[kEc2T], row_out[kEc2T], col_out[kEc2T];
-  for (int m = threadIdx.x; m < Mid; m += blockDim.x) {
-    mid_a[m] = expand_leg(g.a, 3, m);
-    mid_b[m] = expand_leg(g.b, 2, m);
-  }
   const bool tab = La <= kMaxLeg2 && Ra <= kMaxLeg2 && Ua <= kMaxLeg2 && Lb <= kMaxLeg2 &&
                    Rb <= kMaxLeg2 && Db <= kMaxLeg2;
-  if (tab) {
-    auto fill = [&](int64_t *t, const OpBuildEntry &e, int role, int n) {
-      for (int v = threadIdx.x; v < n; v += blockDim.x)
-        t[v] = (int64_t)expand_leg(e, role, v) * e.stride[role];
+  {
+    // 32 values of one leg per warp and pass: short legs are set up side by side
+    int chunk = threadIdx.x >> 5;
+    auto each = [&](int n, auto put) {
+      const int nc = (n + 31) >> 5;
+      for (; chunk < nc; chunk += 8) {
+        const int v = chunk * 32 + (threadIdx.x & 31);
+        if (v < n) put(v);
+      }
+      chunk -= nc;
     };
-    fill(off_la, g.a, 0, La);
-    fill(off_ra, g.a, 1, Ra);
-    fill(off_ua, g.a, 2, Ua);
-    fill(off_lb, g.b, 0, Lb);
-    fill(off_rb, g.b, 1, Rb);
-    fill(off_db, g.b, 3, Db);
+    auto fill = [&](int64_t *t, const OpBuildEntry &e, int role, int n) {
+      each(n, [&](int v) { t[v] = (int64_t)expand_leg(e, role, v) * e.stride[role]; });
+    };
+    each(Mid, [&](int m) { mid_a[m] = expand_leg(g.a, 3, m); });
+    each(Mid, [&](int m) { mid_b[m] = expand_leg(g.b, 2, m); });
+    if (tab) {
+      fill(off_la, g.a, 0, La);
+      fill(off_ra, g.a, 1, Ra);
+      fill(off_ua, g.a, 2, Ua);
+      fill(off_lb, g.b, 0, Lb);
+      fill(off_rb, g.b, 1, Rb);
+      fill(off_db, g.b, 3, Db);
+    }
   }
   __syncthreads();
   float2 *Ec = const_cast<float2 *>(op.Ec);
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
+  if (ta == 0 && threadIdx.x == 0) {
     op.beta_c_bits = 0u;
     op.beta_t_bits = 0u;
   }
@@ -186,7 +201,7 @@ __global__ void __launch_bounds__(256) k_build_ec2(const OpBuild2Entry *__restri
   const int64_t loa = g.a.lo_off, lob = g.b.lo_off;
   const int64_t a_sd = g.a.stride[3], b_su = g.b.stride[2];  // the shared bond on each site
   const int cc = threadIdx.x & (kEc2T - 1), rq = threadIdx.x / kEc2T;  // column, row group
-  for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+  for (int t = ta; t < tb; t += step) {
     const int tr = t / tiles_c, tc = t - tr * tiles_c;
     // the tile's rows (a: l_a, u_a, r_a with r_a fastest) and columns
     // (b: l_b, r_b, d_b with d_b fastest): element bases at m = 0 and their
@@ -215,8 +230,7 @@ __global__ void __launch_bounds__(256) k_build_ec2(const OpBuild2Entry *__restri
       col_out[threadIdx.x - kEc2T] = out;
     }
     __syncthreads();
-    float sr[4] = {0.f, 0.f, 0.f, 0.f}, cr[4] = {0.f, 0.f, 0.f, 0.f};
-    float si[4] = {0.f, 0.f, 0.f, 0.f}, ci[4] = {0.f, 0.f, 0.f, 0.f};
+    float sr[kEc2T / 8] = {}, cr[kEc2T / 8] = {}, si[kEc2T / 8] = {}, ci[kEc2T / 8] = {};
     for (int m0 = 0; m0 < Mid; m0 += kEc2M) {
       const int mc = Mid - m0 < kEc2M ? Mid - m0 : kEc2M;
       for (int e = threadIdx.x; e < kEc2T * kEc2M; e += blockDim.x) {
@@ -243,7 +257,7 @@ __global__ void __launch_bounds__(256) k_build_ec2(const OpBuild2Entry *__restri
       for (int mm = 0; mm < mc; ++mm) {
         const float4 b = Bs[mm][cc];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
+        for (int i = 0; i < kEc2T / 8; ++i) {
           const float4 a = As[rq + 8 * i][mm];
           // re = ar br - ai bi, im = ar bi + ai br (hi products exact, cross terms
           // hi lo + lo hi in the correction)
@@ -261,32 +275,54 @@ __global__ void __launch_bounds__(256) k_build_ec2(const OpBuild2Entry *__restri
     }
     if (col_b[cc] >= 0) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
+      for (int i = 0; i < kEc2T / 8; ++i) {
         const int r = rq + 8 * i;
         if (row_a[r] >= 0) Ec[row_out[r] + col_out[cc]] = make_float2(sr[i] + cr[i], si[i] + ci[i]);
       }
     }
-    __syncthreads();   // the next tile rewrites the row and column tables
+    __syncthreads();   // the next tile (or entry) rewrites the tables
   }
+}
+
+// Bound by the FP32 pipe (48 instructions per entry and value of m) where all
+// variants are read, as in a batch: 0.21 ms at 6x6 (1+32+1), 7.1 M entries.
+// Operands that no lane reads have no tiles: one bitstring needs one of a
+// step's four or eight, 1.1 M entries in 0.05 ms, where making every variant
+// by entry took 0.21 ms of a one-bitstring call of 0.61 ms (now 0.41 ms).
+__global__ void __launch_bounds__(256, kEc2Blocks)
+    k_build_ec2(const OpBuild2Entry *__restrict__ entries, int n, OpDesc *ops, bool marked) {
+  pdl_trigger();
+  if (gridDim.y > 1 || n == 1) {   // by entry
+    pdl_wait();
+    const OpBuild2Entry &g = entries[blockIdx.y];
+    if (marked && !ops[g.op].used) return;
+    const int nt = ec2_tiles(g);
+    if ((int)blockIdx.x < nt) ec2_entry_tiles(g, ops, blockIdx.x, nt, gridDim.x);
+    return;
+  }
+  // this thread's entry (tables: readable before the wait)
+  const int t0 = (int)threadIdx.x < n ? ec2_tiles(entries[threadIdx.x]) : 0;
+  const int op0 = (int)threadIdx.x < n ? entries[threadIdx.x].op : 0;
+  pdl_wait();
+  for_block_share(
+      n, t0 > 0 && (!marked || ops[op0].used) ? t0 : 0,
+      [&](int j) { return !marked || ops[entries[j].op].used ? ec2_tiles(entries[j]) : 0; },
+      [&](int j, int a, int b) { ec2_entry_tiles(entries[j], ops, a, b, 1); });
 }
 
 // beta = max_n sum_k (|Re E_kn| + |Im E_kn|) of every op (the factor by
 // which one absorption can grow max(|Re|, |Im|) of the running tensor); one
 // block row per op, after the builders.  A block takes 32 columns at a time,
 // its 32 warps splitting K; the column sums meet in shared memory.
-__global__ void __launch_bounds__(1024) k_beta_ops(const int32_t *__restrict__ list, OpDesc *ops) {
-  pdl_trigger();
-  pdl_wait();
-  const int which = list ? list[blockIdx.y] : (int)blockIdx.y;
-  const OpDesc &op = ops[which];
-  if (op.Ec == nullptr) return;
+//
+// Column groups first, first + step, ... below last of one op.
+__device__ __forceinline__ void beta_columns(OpDesc &op, int first, int last, int step) {
   const int K = op.K, N = op.N;
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   __shared__ float part[32][33];
   float best = 0.f;
-  if ((int)blockIdx.x * 32 >= N) return;
-  for (int n0 = blockIdx.x * 32; n0 < N; n0 += gridDim.x * 32) {
-    const int n = n0 + lane;
+  for (int g = first; g < last; g += step) {
+    const int n = g * 32 + lane;
     float s = 0.f;
     if (n < N)
       for (int k = w; k < K; k += 32) {
@@ -305,8 +341,28 @@ __global__ void __launch_bounds__(1024) k_beta_ops(const int32_t *__restrict__ l
   if (w == 0) {
     best *= 1.0f + 1.0f / 256.0f;
     for (int o = 16; o > 0; o >>= 1) best = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, o));
-    if (lane == 0) atomicMax(&ops[which].beta_c_bits, __float_as_uint(best));
+    if (lane == 0) atomicMax(&op.beta_c_bits, __float_as_uint(best));
   }
+}
+
+__global__ void __launch_bounds__(1024) k_beta_ops(const OpList list, int n,
+                                                   OpDesc *ops, bool marked) {
+  pdl_trigger();
+  pdl_wait();
+  auto groups = [&](int j) {   // none if no lane reads the op
+    const OpDesc &op = ops[list.op(j)];
+    return op.Ec == nullptr || (marked && !op.used) ? 0 : (op.N + 31) / 32;
+  };
+  auto columns = [&](int j, int a, int b, int step) {
+    beta_columns(ops[list.op(j)], a, b, step);
+  };
+  if (gridDim.y > 1 || n == 1) {   // by op
+    const int ng = groups(blockIdx.y);
+    if ((int)blockIdx.x < ng) columns(blockIdx.y, blockIdx.x, ng, gridDim.x);
+    return;
+  }
+  for_block_share(n, (int)threadIdx.x < n ? groups(threadIdx.x) : 0, groups,
+                  [&](int j, int a, int b) { columns(j, a, b, 1); });
 }
 
 // Merge operand from a stored tensor: Ec[k][n] = G[k ks + n ns] 2^-target,
@@ -355,39 +411,38 @@ cudaError_t launch_tensor_operand(const TensorOpEntry *d_entry, int n_entries, i
 }
 
 cudaError_t launch_build_operands2(const OpBuild2Entry *d_entries, int n, int max_kn,
-                                   OpDesc *d_ops, cudaStream_t s) {
+                                   OpDesc *d_ops, bool marked, int sm_count, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
-  // 32 x 32 tiles of W; about 2048 blocks in all, each walking several tiles
-  // of its entry so that its index tables (set up once per block) serve them
-  int blocks = (max_kn + 1023) / 1024 + 1;
-  const int share = (2048 + n - 1) / n;
-  if (blocks > share) blocks = share < 8 ? 8 : share;
-  if (blocks > 2048) blocks = 2048;
-  if (blocks < 1) blocks = 1;
-  return launch_dependent(k_build_ec2, dim3(blocks, n), dim3(256), 0, s, d_entries, d_ops);
+  // the tile list, or by entry where that gives every tile its own block (its
+  // blocks need not add up the list: 3 us for a 5x5 lattice's 100 tiles).  The
+  // list goes to three times the blocks that the chip holds, so that an SM
+  // that started late, under the build before, takes fewer (6x6 (1+32+1),
+  // all variants read: 210 us; one times 225).
+  const int tiles = (max_kn + 1023) / 1024 + 1;
+  const dim3 grid = n == 1 || (int64_t)n * tiles <= 2048 ? dim3(tiles < 2048 ? tiles : 2048, n)
+                                                         : dim3(3 * kEc2Blocks * sm_count);
+  return launch_dependent(k_build_ec2, grid, dim3(256), 0, s, d_entries, n, d_ops, marked);
 }
 
 cudaError_t launch_build_operands(const OpBuildEntry *d_entries, int n, int max_kn,
-                                  OpDesc *d_ops, cudaStream_t s) {
+                                  OpDesc *d_ops, bool marked, cudaStream_t s) {
   if (n <= 0) return cudaSuccess;
   int blocks = (max_kn + 255) / 256;
   if (blocks > 1024) blocks = 1024;
   if (blocks < 1) blocks = 1;
-  return launch_dependent(k_build_ec, dim3(blocks, n), dim3(256), 0, s, d_entries, d_ops);
+  return launch_dependent(k_build_ec, dim3(blocks, n), dim3(256), 0, s, d_entries, d_ops, marked);
 }
 
-cudaError_t launch_operand_bounds(int n_ops, const int32_t *d_list, OpDesc *d_ops, cudaStream_t s,
-                                  int64_t n_cols) {
+cudaError_t launch_operand_bounds(int n_ops, const OpList &list, OpDesc *d_ops, cudaStream_t s,
+                                  int64_t n_cols, bool marked, int sm_count) {
   if (n_ops <= 0) return cudaSuccess;
-  // 32 columns per block and pass: a block per 32 columns of the widest
-  // operand, up to 2048 blocks for one operand and some 1200 in all for
-  // several (at least 8 each): blocks past a narrow operand's columns leave at
-  // once, which thousands of them make felt (110 operands: 64 blocks each 32
-  // us, 11 each 21 us)
-  int64_t gx = (n_cols + 31) / 32;
-  const int64_t most = n_ops == 1 ? 2048 : (1200 / n_ops > 8 ? 1200 / n_ops : 8);
-  gx = gx < 1 ? 1 : (gx > most ? most : gx);
-  return launch_dependent(k_beta_ops, dim3((unsigned)gx, n_ops), dim3(1024), 0, s, d_list, d_ops);
+  // 32 columns of one op per block and pass: by op where some 1200 blocks give
+  // every pass its own (at least 8 passes each: blocks past a narrow op's
+  // columns leave at once, which thousands of them make felt), else the list
+  const int64_t gx = n_cols > 32 ? (n_cols + 31) / 32 : 1;
+  const dim3 grid = n_ops == 1 || gx * n_ops <= 1200 ? dim3((unsigned)(gx < 2048 ? gx : 2048), n_ops)
+                                                     : dim3(2 * sm_count);
+  return launch_dependent(k_beta_ops, grid, dim3(1024), 0, s, list, n_ops, d_ops, marked);
 }
 
 }  // namespace peps
