@@ -152,6 +152,7 @@ struct Plan {
   int n_site_ops = 0;           // ops rebuilt from the site tensors per slice
   int64_t max_kn_merge = 0;
   size_t off_tops = 0, off_dots = 0, off_partials = 0;
+  size_t partials = 0;          // entries at off_partials
   int bufs_per_lane = 2;
   std::vector<int> step_site;
   std::vector<int> step_opbase;  // first OpDesc of each step (2^nq variants)
@@ -1973,13 +1974,14 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
   P.off_partials = off;
   {
     // per lane: the separate dot kernel's blocks, or a fused merge's slots
-    // (at most ceil(M / 128) x (2N / 16) tiles x 4 warps)
     size_t per_lane = kDotBlocks;
     if (quad && !P.odd) {
       const StepShape &m2 = P.steps[P.s_m2];
-      per_lane = std::max(per_lane, (size_t)((m2.M + 127) / 128) * (size_t)(2 * m2.N / 16) * 4);
+      if (want_tc && tc_supports(m2, fmt))
+        per_lane = std::max(per_lane, (size_t)tc_dot_slots(m2, fmt, o.tc_kchunk, o.tc_epi));
     }
-    off = align_up(off + (quad ? per_lane * P.lanes * sizeof(double2) : 16));
+    P.partials = quad ? per_lane * P.lanes : 1;
+    off = align_up(off + P.partials * sizeof(double2));
   }
   P.off_small_steps = off;
   off = align_up(off + (size_t)std::max(NS, (int64_t)1) *
@@ -2041,8 +2043,11 @@ static int build_plan(peps_ctx *c, int64_t n, const peps_opts &o, const void *ws
   // fused dots: the merge's partial-sum slots per item
   for (auto &l : P.launches) {
     if (l.kind != 3 || l.fused_merge < 0) continue;
-    const int slots = tc_dot_slots(P.launches[l.fused_merge].tc_handle);
-    for (int k = 0; k < l.n_aux; ++k) dots[l.aux_off + k].nslots = slots;
+    const int64_t slots = tc_dot_slots(P.launches[l.fused_merge].tc_handle);
+    if (slots * l.n_aux > (int64_t)P.partials || slots > INT32_MAX)
+      return fail(PEPS_EINVAL, "internal: %lld partial sums of %d lanes, room for %zu",
+                  (long long)slots, l.n_aux, P.partials);
+    for (int k = 0; k < l.n_aux; ++k) dots[l.aux_off + k].nslots = (int32_t)slots;
   }
 
   std::vector<OpDesc> ops(n_ops);

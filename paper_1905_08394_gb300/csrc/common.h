@@ -434,8 +434,10 @@ cudaError_t launch_contract_tc(void *handle, const StepItem *d_items, int n_item
                                const OpDesc *d_ops, Rec *d_recs, DeviceStatus *st,
                                int64_t watchdog_ns, int sm_count, cudaStream_t s,
                                double2 *dot_partials = nullptr);
-// Partial-sum slots per item of a fused-dot launch (sh.dot).
-int tc_dot_slots(const void *handle);
+// Partial-sum slots per item of a fused-dot launch: of a step with the tuning
+// that tc_prepare gets (to size the workspace), and of what it prepared.
+int64_t tc_dot_slots(const StepShape &sh, int fmt, int kchunk, int epi);
+int64_t tc_dot_slots(const void *handle);
 int tc_Kr_pad(int K);   // real K of a tensor-core operand
 int tc_Nr_pad(int N);   // real N
 

@@ -1115,6 +1115,39 @@ bool tc_supports(const StepShape &sh, int fmt) {
   return true;
 }
 
+// Accumulators and column width of a step's tiles, before what the launch
+// (its items, its buffers' alignment) makes of them.
+struct TileCols {
+  int ksplit, csep;   // K segments, a correction accumulator (0 or 1)
+  int BN;
+};
+static TileCols tile_cols(const StepShape &sh, int np, int kb_count) {
+  const int Nr = 2 * sh.N;
+  // K segments (long-K steps): at most one per k-chunk
+  int KS = sh.ksplit > 1 ? sh.ksplit : 1;
+  if (KS > kb_count) KS = kb_count;
+  const int CS = (sh.csep && np == 2) ? 1 : 0;
+  const int NA = KS + CS;
+  // BN: the widest tile that divides Nr in whole 16-column chunks and whose NA
+  // accumulators fit TMEM (twice where K is short, at most 16 k-chunks, which
+  // needs the epilogue overlap of two buffers)
+  const int cols_max = 512 / (kb_count <= 16 ? 2 * NA : NA);
+  int BN = Nr < 256 ? Nr : 256;
+  if (BN > cols_max) BN = cols_max / 16 * 16;
+  while (BN > 16 && Nr % BN != 0) BN -= 16;
+  return {KS, CS, BN};
+}
+
+// A fused dot keeps the width of tile_cols and takes eight epilogue warps unless
+// four are asked for; every warp of every tile writes a slot, with columns of
+// its own or not.
+int64_t tc_dot_slots(const StepShape &sh, int fmt, int kchunk, int epi) {
+  const int esz = esz_of(fmt), Kr = 2 * sh.K, rowb = rowb_for(Kr, esz, kchunk);
+  if (!rowb) return 0;
+  const int BN = tile_cols(sh, np_of(fmt), Kr * esz / rowb).BN;
+  return ((sh.M + BM - 1) / BM) * (2 * sh.N / BN) * (epi == 4 ? 4 : 8);
+}
+
 struct TcLaunchData {
   TcParams prm;
   int rowb;
@@ -1219,20 +1252,10 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
       return -3;
     }
   }
-  // K segments (long-K steps): at most one per k-chunk, and BN small enough
-  // that KS accumulators are double-buffered within TMEM's 512 columns
   const int kb_count = (Kr * esz) / rowb;
-  int KS = sh.ksplit > 1 ? sh.ksplit : 1;
-  if (KS > kb_count) KS = kb_count;
-  const int CS = (sh.csep && np == 2) ? 1 : 0;
-  const int NA = KS + CS;
-  // BN: the widest tile that divides Nr in whole 16-column chunks and whose NA
-  // accumulators fit TMEM (twice where K is short, at most 16 k-chunks, which
-  // needs the epilogue overlap of two buffers)
-  const int cols_max = 512 / (kb_count <= 16 ? 2 * NA : NA);
-  int BN = Nr < 256 ? Nr : 256;
-  if (BN > cols_max) BN = cols_max / 16 * 16;
-  while (BN > 16 && Nr % BN != 0) BN -= 16;
+  const TileCols tc = tile_cols(sh, np, kb_count);
+  const int KS = tc.ksplit, CS = tc.csep, NA = KS + CS;
+  int BN = tc.BN;
   // entries in contiguous runs of 8 (the epilogue's W = 8)
   const int run = sh.vb && sh.nvs ? sh.dh_out : (sh.dv_out == 1 && sh.P == 1 ? sh.N : sh.dv_out);
   const bool runs8 = !sh.dot && run % 8 == 0 && (sh.vb ? sh.nvs && sh.P == 1 : true);
@@ -1463,9 +1486,9 @@ cudaError_t tc_warm(void *handle) {
   return with_kernel_of((const TcLaunchData *)handle, WarmKernel{});
 }
 
-int tc_dot_slots(const void *handle) {
+int64_t tc_dot_slots(const void *handle) {
   const TcLaunchData *d = (const TcLaunchData *)handle;
-  return d->prm.tiles_m * d->prm.tiles_n * d->epi;
+  return (int64_t)d->prm.tiles_m * d->prm.tiles_n * d->epi;
 }
 
 cudaError_t launch_contract_tc(void *handle, const StepItem *d_items, int n_items,
