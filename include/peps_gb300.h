@@ -175,7 +175,8 @@ typedef struct {
     int32_t tc_cluster;       /* tensor-core tuning: 2 = CTA pairs compute
                                  256-row tiles with the 2-SM MMA, 1 = one CTA
                                  per 128-row tile (0 = pairs where the row
-                                 tiles pair up)                              */
+                                 tiles pair up; either way only for tiles of
+                                 a multiple of 32 real columns)              */
     int32_t fuse_rows;        /* contraction order: 0 = absorb the two top and
                                  the two bottom rows of a column in one step
                                  each where that costs no more multiply-adds

@@ -31,9 +31,9 @@
 // TB/s); of a 4096 x 64 x 512 step: 172 -> 61 us; the open-leg step 32768 x 128
 // x 256 with P = 16, one item: 155 -> 38 us.
 //
-// CG = 2 (the default where the row tiles pair up): a cluster of two CTAs on
-// neighbouring SMs computes a 256-row tile with the 2-SM UMMA
-// (tcgen05.mma.cta_group::2, M = 256).  Each CTA loads its own 128 rows of A
+// CG = 2 (the default where the row tiles pair up and BN is a multiple of 32): a
+// cluster of two CTAs on neighbouring SMs computes a 256-row tile with the 2-SM
+// UMMA (tcgen05.mma.cta_group::2, M = 256).  Each CTA loads its own 128 rows of A
 // and only half of the Bt tile; the even CTA issues the MMAs for both, and
 // the TMA completions of both CTAs arrive on its barriers.  Per SM this
 // halves the Bt bytes ingested per multiply-add, which is what bounds the
@@ -1273,15 +1273,15 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
               : runs8 && (sh.M / 256) * (Nr / 256) * (int64_t)n_items >= (BN == 256 ? 38 : 152));
   if (drain) BN = 256;
   // A launch of fewer tiles than CTA pairs is as long as one tile: narrower
-  // tiles (down to 64 columns) put more SMs on it.  One item of 256 x 1024 x
+  // tiles (down to 64 columns, in whole 32s for the pairs) put more SMs on it.  One item of 256 x 1024 x
   // 1024: 38.9 -> 32.7 us, of 1024 x 128 x 512: 15.9 -> 12.4 us.
   const int64_t row_tiles = (sh.M + 2 * BM - 1) / (2 * BM);
-  while (!drain && !sh.dot && BN > 64 && BN % 32 == 0 && row_tiles * (Nr / BN) * n_items < 76)
+  while (!drain && !sh.dot && BN >= 128 && BN % 64 == 0 && row_tiles * (Nr / BN) * n_items < 76)
     BN /= 2;
   const int tiles_m = (int)((sh.M + BM - 1) / BM);
-  // The 2-SM UMMA when the 128-row tiles pair up and each CTA's half of the
-  // Bt tile is a whole number of 8-row swizzle groups.
-  d->cg = ((BN / 2) % 8 == 0 && tiles_m % 2 == 0 && cluster != 1) ? 2 : 1;
+  // The 2-SM UMMA when the 128-row tiles pair up and the columns are a multiple
+  // of 32, as its M = 256 form is specified for (the one-CTA form: of 16).
+  d->cg = (BN % 32 == 0 && tiles_m % 2 == 0 && cluster != 1) ? 2 : 1;
   // B: one map per plane over every operand variant {k, n, variant}; the
   // variants are equally spaced (a single variant gets the packed stride)
   const int64_t bpacked = (int64_t)Kr * esz * Nr;

@@ -45,6 +45,11 @@ cudaError_t launch(const void *f, dim3 grid, dim3 block, void **args, size_t sme
     line(" %llu", v);
   }
   g_log += '\n';
+  if (name.find("k_store_out") != std::string::npos) {   // the status words, which the host reads
+    const void *st = *(const void **)args[3];
+    void *tail = *(void **)args[4];
+    if (tail) std::memcpy(tail, st, 16);
+  }
   return cudaSuccess;
 }
 
