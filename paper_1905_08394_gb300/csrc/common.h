@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <atomic>
 #include <string>
 #include <vector>
 
@@ -72,6 +73,40 @@ inline Div make_div(int64_t d) {
   while (((int64_t)1 << v.l) < (int64_t)v.d) ++v.l;
   v.m = (uint32_t)(((((uint64_t)1 << v.l) - v.d) << 32) / v.d + 1);
   return v;
+}
+
+// What a kernel needs once on each device before it runs there: f(&value) on
+// the first call with that device current (a failure is not kept, so the next
+// call tries again), its value (>= 0) from then on.  A function attribute
+// belongs to one device, so a flag for the whole process would leave the others
+// without it.
+constexpr int kMaxDevices = 64;
+struct PerDevice {
+  std::atomic<int> done[kMaxDevices];   // value + 1; 0: not yet
+  template <class F>
+  cudaError_t get(int *value, F f) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    const bool kept = dev >= 0 && dev < kMaxDevices;
+    const int v = kept ? done[dev].load(std::memory_order_acquire) : 0;
+    if (v > 0) {
+      *value = v - 1;
+      return cudaSuccess;
+    }
+    e = f(value);
+    if (e == cudaSuccess && kept) done[dev].store(*value + 1, std::memory_order_release);
+    return e;
+  }
+};
+// The same for a kernel's shared-memory limit alone.
+template <class K>
+inline cudaError_t allow_smem(PerDevice &state, K kern, size_t bytes) {
+  int unused = 0;
+  return state.get(&unused, [&](int *v) {
+    *v = 0;
+    return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+  });
 }
 
 // ---------------------------------------------------------------------------

@@ -419,8 +419,8 @@ cudaError_t launch_cfg(const SimtParams &p, const StepItem *items, int n_items, 
   constexpr size_t smem = 2 * ROWS * (BK + 2) * sizeof(float2) + 2 * 3 * BK * COLS * sizeof(float);
   auto kern = k_contract_simt<FMT, RT, CT, WN, BK>;
   if (smem > 48 * 1024) {
-    static const cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    static PerDevice allowed;
+    const cudaError_t e = allow_smem(allowed, kern, smem);
     if (e != cudaSuccess) return e;
   }
   int64_t mt = (p.sh.M + ROWS - 1) / ROWS;

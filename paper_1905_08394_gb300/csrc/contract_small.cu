@@ -200,14 +200,9 @@ SmallStep small_step(const StepShape &sh) {
 cudaError_t launch_sweep_small(const SmallSweep &p, int sm_count, cudaStream_t s) {
   if (p.n <= 0) return cudaSuccess;
   const size_t smem = small_sweep_smem(p.cap_g, p.cap_e);
-  static int configured = 0;   // dynamic shared memory above 48 KiB needs the opt-in
-  if (!configured) {
-    cudaError_t e = cudaFuncSetAttribute(k_sweep_small,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)kSmallSweepMaxSmem + 512);   // padding of the parts
-    if (e != cudaSuccess) return e;
-    configured = 1;
-  }
+  static PerDevice allowed;   // (padding of the parts)
+  const cudaError_t e = allow_smem(allowed, k_sweep_small, kSmallSweepMaxSmem + 512);
+  if (e != cudaSuccess) return e;
   if (smem > kSmallSweepMaxSmem + 512) return cudaErrorInvalidValue;
   // blocks resident per SM (about 220 KiB of shared memory), at most 4
   const int per_sm = (int)((220u * 1024u) / (smem > 0 ? smem : 1));

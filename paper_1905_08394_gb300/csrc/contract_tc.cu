@@ -1372,17 +1372,13 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
 
 void tc_release(void *h) { delete (TcLaunchData *)h; }
 
+// The kernel set up on the current device; *max_clusters: co-resident clusters
+// at the largest shared-memory size (0: not known).
 template <int FMT, int ROWB, int CG, int EPI, int DR>
-static int &max_clusters_of() {
-  static int v = -1;  // co-resident clusters at the largest smem size (-1: not set up)
-  return v;
-}
-
-template <int FMT, int ROWB, int CG, int EPI, int DR>
-static cudaError_t init_kernel() {
-  auto kern = k_contract_tc<FMT, ROWB, CG, EPI, DR>;
-  int &max_clusters = max_clusters_of<FMT, ROWB, CG, EPI, DR>();
-  if (max_clusters < 0) {
+static cudaError_t init_kernel(int *max_clusters) {
+  static PerDevice state;
+  return state.get(max_clusters, [](int *n) {
+    auto kern = k_contract_tc<FMT, ROWB, CG, EPI, DR>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          227 * 1024);
     if (e != cudaSuccess) return e;
@@ -1397,23 +1393,22 @@ static cudaError_t init_kernel() {
     q.dynamicSmemBytes = 227 * 1024;
     q.attrs = qa;
     q.numAttrs = 1;
-    int n = 0;
-    e = cudaOccupancyMaxActiveClusters(&n, (void *)kern, &q);
-    if (e != cudaSuccess || n <= 0) {
+    *n = 0;
+    e = cudaOccupancyMaxActiveClusters(n, (void *)kern, &q);
+    if (e != cudaSuccess || *n <= 0) {
       (void)cudaGetLastError();
-      n = 0;
+      *n = 0;
     }
-    max_clusters = n;
-  }
-  return cudaSuccess;
+    return cudaSuccess;
+  });
 }
 
 template <int FMT, int ROWB, int CG, int EPI, int DR>
 static cudaError_t launch_one(const TcParams &prm, int units, size_t smem, cudaStream_t s) {
   auto kern = k_contract_tc<FMT, ROWB, CG, EPI, DR>;
-  cudaError_t e0 = init_kernel<FMT, ROWB, CG, EPI, DR>();
+  int max_clusters = 0;
+  const cudaError_t e0 = init_kernel<FMT, ROWB, CG, EPI, DR>(&max_clusters);
   if (e0 != cudaSuccess) return e0;
-  const int max_clusters = max_clusters_of<FMT, ROWB, CG, EPI, DR>();
   // units = SMs to use; one CTA per SM, clusters of CG
   int clusters = units / CG;
   if (max_clusters > 0 && clusters > max_clusters) clusters = max_clusters;
@@ -1471,7 +1466,10 @@ static cudaError_t with_kernel_of(const TcLaunchData *d, F f) {
 }
 struct WarmKernel {
   template <int FMT, int ROWB, int CG, int EPI, int DR>
-  cudaError_t run() const { return init_kernel<FMT, ROWB, CG, EPI, DR>(); }
+  cudaError_t run() const {
+    int unused = 0;
+    return init_kernel<FMT, ROWB, CG, EPI, DR>(&unused);
+  }
 };
 struct LaunchKernel {
   const TcParams &prm;

@@ -17,7 +17,7 @@ std::map<const void *, std::string> &names() {   // host stub -> device name
   return *m;
 }
 std::map<std::pair<int, const void *>, int> g_smem;   // (device, kernel) -> dynamic limit
-int g_device = 0;
+int g_device = 0, g_refuse = 0;
 dim3 g_grid, g_block;
 size_t g_shared;
 void *g_stream;
@@ -68,6 +68,7 @@ CUresult encode(CUtensorMap *, CUtensorMapDataType, cuuint32_t rank, void *base,
 FAKE const char *fake_log() { return g_log.c_str(); }
 FAKE void fake_clear() { g_log.clear(); }
 FAKE void fake_set_device(int d) { g_device = d; }
+FAKE void fake_refuse_attributes(int n) { g_refuse = n; }   // the next n times
 
 // what compiled CUDA code registers and launches through
 FAKE void **__cudaRegisterFatBinary(void *) { static void *h; return &h; }
@@ -106,6 +107,7 @@ FAKE cudaError_t cudaLaunchKernelExC(const cudaLaunchConfig_t *c, const void *f,
   return launch(f, c->gridDim, c->blockDim, args, c->dynamicSmemBytes, cluster);
 }
 FAKE cudaError_t cudaFuncSetAttribute(const void *f, cudaFuncAttribute a, int v) {
+  if (g_refuse > 0 && g_refuse--) return cudaErrorInvalidValue;
   if (a == cudaFuncAttributeMaxDynamicSharedMemorySize) g_smem[{g_device, f}] = v;
   return cudaSuccess;
 }
