@@ -13,7 +13,8 @@ value   amplitudes/s of the mixed-precision path (FP16 hi/lo split, three
         tensor-core products, FP32 accumulate), bitstrings resident in HBM,
         CUDA events around the timed steps on the launch stream.
 e2e     the same through the host C-ABI call (pinned host bitstrings copied
-        in, amplitudes copied out, inside the timed region).
+        in, amplitudes copied out by way of the context, inside the timed
+        region).
 fp32_path  the plain FP32 CUDA-core form on the same GPU (timed on one group
         of 64 bitstrings; the work per amplitude is identical across groups).
 square_partition  the same batch contracted by the square partition of the
@@ -88,7 +89,7 @@ def golden_check(out, bits, first=0):
 # per launch is this ratio times its own algorithmic bytes per launch: the
 # same steps, with more lanes per launch, and traffic in proportion to the
 # lanes.  Valid while the kernel's sources hash to the captured version.
-TRAFFIC = {"sources_sha256_16": "99a6e6e12e7c04e0", "dram_per_algorithmic_byte": 0.836}
+TRAFFIC = {"sources_sha256_16": "3e263fc0ad3239bb", "dram_per_algorithmic_byte": 0.680}
 TRAFFIC_SOURCES = ("contract_tc.cu", "common.h", "format.cuh")
 
 

@@ -26,11 +26,12 @@
 // += a.y b.x, k ascending).  The packed form halves the issue slots: with
 // distinct operands it reaches 60 TFLOP/s on its own, and this kernel is 14 %
 // faster with it than with scalar multiply-adds.  Large K is bound by that rate,
-// small K by memory, launches of few tiles by latency.  The 4 x 8 tiles, at 47
-// TFLOP/s, keep 64 sums per thread: at the 128 registers that two blocks per SM
-// leave, ptxas spills 92 to 204 bytes a thread, and the operand lies in three
-// planes in shared memory (b.y and -b.y both).  What either costs has not been
-// measured apart.
+// small K by memory, launches of few tiles by latency.  The 4 x 8 tiles (42 to
+// 51 TFLOP/s on the square partition's large steps at 64 lanes) keep 64 sums per
+// thread: at the 128 registers that two blocks per SM leave, ptxas spills 92 to
+// 204 bytes a thread, and the operand lies in three planes in shared memory (b.y
+// and -b.y both).  What either costs has not been measured apart; the 2 x 8 tile
+// with K passes of 16, which spills nothing, reaches 47.
 #include "common.h"
 #include "format.cuh"
 
