@@ -1263,8 +1263,8 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
   // 256-column tiles.  For a short K that is the alternative to 128-column
   // tiles with two buffers, which load every row of A twice as often: 16 lanes
   // of 65536 x 256 x 256 took 1408 us that way, at 9 TB/s from L2 into shared
-  // memory; 1072 us now (512 lanes of the fused 1024 x 1024 x 256 merge: 1912 ->
-  // 1756 us).  It needs tiles for every CTA pair; the fused dot's
+  // memory; 1072 us drained, 993 with the interleaved order below as well (512
+  // lanes of the fused 1024 x 1024 x 256 merge: 1912, 1756, 1632 us).  It needs tiles for every CTA pair; the fused dot's
   // tiles keep their width (it fixes the order of its partial sums).
   const bool wide32 = (uintptr_t)a_base % 32 == 0;
   const bool drain =
@@ -1357,10 +1357,11 @@ int tc_prepare(const StepShape &sh, int fmt, const void *a_base, int a_lanes,
   // tiles of at least 64 columns, K <= 32 on 32) and where it is not hidden at
   // all (one accumulator buffer: the merges; the fused dot), four where the
   // MMAs do or where a second warp per quadrant finds no columns.  Measured,
-  // eight / four warps: 16 lanes of 4096 x 64 x 512 60.6 / 69.7 us, 65536 x 16 x
-  // 256 518 / 678 us, 4096^3 merge 11.43 / 11.60 ms; 65536 x 256 x 256 1408 /
-  // 1382 us, 512 lanes of 1024 x 128 x 512 584 / 549 us, 32768 x 64 x 8 66.0 /
-  // 61.7 us.
+  // eight / four warps: 16 lanes of 65536 x 16 x 256 446 / 460 us, of 4096 x 64 x
+  // 512 58.6 / 59.3 us (BF16 36.1 / 38.1), one item of 256 x 1024 x 1024 49.5 / 59.0
+  // us; 512 lanes of 1024 x 128 x 512 537 / 518 us, 16 of 32768 x 64 x 8 64.8 / 61.7
+  // us.  (Drained against four warps: the fused 1024 x 1024 x 256 merge of 512
+  // lanes 1632 / 1932 us, 16 lanes of 65536 x 256 x 256 993 / 1366 us.)
   const bool epi_bound = sh.dot || d->prm.nbuf == 1 || (sh.K <= 64 && BN >= 64) ||
                          (sh.K <= 32 && BN >= 32);
   d->epi = epi == 4 || epi == 8 ? epi : (epi_bound ? 8 : 4);
